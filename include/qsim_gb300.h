@@ -106,7 +106,9 @@ typedef struct sim_plan_opts {
                                 Ozaki, Ogita, Oishi and Rump 2012); each result is within about
                                 2^-42 of its row's and column's largest entries at worst (2^-47 for
                                 the fixed-point rounding).  Every fused plan needs
-                                n >= k + 7 (SIM_EINVAL otherwise). */
+                                n >= k + 7 (SIM_EINVAL otherwise).  Large registers (k = 6 from 26
+                                qubits, complex128 from 22): stretches of a unitary circuit that
+                                are predicted to be faster in register tiles run as tile passes. */
     int32_t tile_qubits;     /* SIM_PLAN_STAGED: tile size log2 (0 = default) */
     int32_t flags;           /* SIM_FLAG_* bits, 0 = defaults */
 } sim_plan_opts;
@@ -297,7 +299,7 @@ int sim_batch_create(int count, const int32_t *n_qubits, const int64_t *gate_off
  *   tile_qubits in {0, 11, 12, 13} (0 = 13): qubits per register tile (a
  *   circuit of up to that many qubits lives in one CTA; larger ones run tile
  *   passes over a scratch state); ctas_per_sm >= 0 (0 = as many as fit: two
- *   with 13-qubit tiles, three with 11 or 12): persistent CTAs per SM.
+ *   with 13-qubit tiles, four with 12, six with 11): persistent CTAs per SM.
  *   SIM_EINVAL outside those ranges or above what fits.
  * sim_batch_config: the configuration a batch uses, its algorithmic flops
  *   (8 per complex multiply-add of the gates as given, summed over the
@@ -336,7 +338,11 @@ int sim_batch_destroy(sim_batch_t b);
  *   eps 1e-8, learning rate lr); *final_loss (may be NULL) after the last.
  * sim_set_cost_model: SIM_PLAN_LEARNED on this handle consults model m (NULL
  *   = no model: the greedy fixed-k plan is used).  The model must outlive the
- *   handle's use of it.  A complex128 handle runs SIM_PLAN_LEARNED without
+ *   handle's use of it.  Registers of 12 to 25 qubits run 12-qubit register
+ *   tiles without asking it (fastest, or within 3 %, on every circuit family;
+ *   asking costs more than that); from 26 qubits on it is asked about the windows that
+ *   controlled exchanges decide, the others run as the fused plan with k = 6,
+ *   which takes tile passes where they are faster.  A complex128 handle runs SIM_PLAN_LEARNED without
  *   consulting the model (trained on complex64 timings): as the fused plan
  *   with k = 4 when n >= 11 (tensor-core digit products; the per-gate and
  *   register-tile kernels are bound by the FP64 pipe), else per gate. */
@@ -376,15 +382,18 @@ int sim_last_plan(sim_t s, int32_t *variants, size_t cap, size_t *len);
  *   With opts->plan = SIM_PLAN_FUSED (fuse_k 0 = 5): *passes gets the passes
  *   the fused plan makes over the state (a multi-block pass counts once,
  *   see SIM_FLAG_MULTI_BLOCK_PASSES),
- *   *ops the fused blocks; *layout_changes and *order_len are set to 0.
+ *   *ops the fused blocks, if all of it runs in blocks; *layout_changes and
+ *   *order_len are set to 0.
  *   Other plans: SIM_EUNSUPPORTED. */
 int sim_plan_describe(int n, int dtype, const sim_gate *gates, size_t n_gates, const sim_plan_opts *opts,
                       int64_t *passes, int64_t *ops, int64_t *layout_changes, int32_t *order, size_t order_cap,
                       size_t *order_len);
 
-/* sim_plan_staged_ops: the SIM_PLAN_STAGED encoding of a circuit, host only,
+/* sim_plan_staged_ops: the SIM_PLAN_STAGED schedule of a circuit, host only,
  *   for inspection and for checking the planner without a GPU (the record
- *   layout follows the library's version).  A tile is 2^M amplitudes: local
+ *   layout follows the library's version): which gates each pass applies, and
+ *   one valid order and layout for them.  What the kernels run is compiled
+ *   from the passes (sim_plan_tile_programs).  A tile is 2^M amplitudes: local
  *   bits 0..4 are qubits 0..4, local bit 5 + i is the pass's high qubit i;
  *   256 threads hold 2^(M - 8) registers each.  Register layout l places
  *   register bit j and thread bit i on local bits given by the library's
@@ -418,6 +427,20 @@ typedef struct sim_tile_op {
 #define SIM_TILE_PASS_INFO 24
 int sim_plan_staged_ops(int n, int dtype, const sim_gate *gates, size_t n_gates, int tile_qubits, sim_tile_op *ops,
                         size_t ops_cap, int32_t *info, size_t info_cap, size_t *n_ops, size_t *n_passes);
+
+/* sim_plan_tile_programs: the tile programs of a SIM_PLAN_STAGED circuit -- what the
+ *   register-tile kernels execute -- host only, with FP64 tables, for checking
+ *   the compiler without a GPU (operations and their encoding: the head of
+ *   csrc/tileprog.cuh).  words: up to words_cap 32-bit words of all passes;
+ *   info: SIM_TILE_PASS_INFO int32 per pass (first word, word count, M,
+ *   register bits, amplitudes per I/O vector, the layouts the pass loads and
+ *   stores in, the low and high half of the mask of qubits whose labels the
+ *   store exchanges, the number of high qubits, the high qubits); *n_words,
+ *   *n_passes the full counts (a pass of diagonal gates alone vanishes into
+ *   the next; SWAPs without controls rename the qubits of later gates, and the
+ *   last passes bring them back).  SIM_EINVAL if no tile fits or a gate is invalid. */
+int sim_plan_tile_programs(int n, int dtype, const sim_gate *gates, size_t n_gates, int tile_qubits, uint32_t *words,
+                           size_t words_cap, int32_t *info, size_t info_cap, size_t *n_words, size_t *n_passes);
 
 /* ---- instrumentation --------------------------------------------------------
  * sim_profile_enable: when on, every kernel launch of the handle is bracketed

@@ -463,6 +463,21 @@ int sim_plan_staged_ops(int n, int dtype, const sim_gate *gates, size_t n_gates,
     return encode_staged(n, dtype, gates, n_gates, tile_qubits, ops, ops_cap, info, info_cap, n_ops, n_passes);
 }
 
+int sim_plan_tile_programs(int n, int dtype, const sim_gate *gates, size_t n_gates, int tile_qubits, uint32_t *words,
+                           size_t words_cap, int32_t *info, size_t info_cap, size_t *n_words, size_t *n_passes)
+{
+    set_error("");
+    if (n < 1 || n > 34) return fail(SIM_EINVAL, "sim_plan_tile_programs: n must be in [1, 34]");
+    if (dtype != SIM_C64 && dtype != SIM_C128) return fail(SIM_EINVAL, "sim_plan_tile_programs: bad dtype");
+    if (n_gates && !gates) return fail(SIM_EINVAL, "sim_plan_tile_programs: gates is NULL");
+    for (size_t k = 0; k < n_gates; ++k) {
+        std::string why;
+        if (validate_gate(n, gates[k], &why)) return fail(SIM_EINVAL, "sim_plan_tile_programs: " + why);
+    }
+    return export_tile_programs(n, dtype, gates, n_gates, tile_qubits, words, words_cap, info, info_cap, n_words,
+                                n_passes);
+}
+
 int sim_profile_enable(sim_t s, int on)
 {
     if (int rc = check_handle(s)) return rc;

@@ -25,7 +25,7 @@
 #include <numeric>
 #include <vector>
 
-#include "tile.cuh"
+#include "tileprog.cuh"
 
 struct qsim_batch;
 
@@ -47,9 +47,11 @@ struct BCirc {
 };
 
 struct BPass {
-    int64_t op0;
-    int32_t nops;
+    int64_t prog0;        // first 16-byte unit of its tile program
+    int32_t nunits;
     int32_t need;         // tiles of the previous pass that must be stored first
+    int32_t start_layout, end_layout;
+    uint64_t flip;        // qubits whose labels the last operation leaves exchanged
     TileGeom geo;
 };
 
@@ -79,20 +81,19 @@ __global__ void k_batch_reset(BCtl *ctl, int *done, int64_t ndone, int *finished
     for (int64_t j = i; j < ncirc; j += stride) finished[j] = 0;
 }
 
-// tiles of up to 12 qubits fit three CTAs per SM (as the staged plan's),
-// 13-qubit tiles two
-template <int M>
-__global__ void __launch_bounds__(kThr, M <= 12 ? 3 : 2)
+template <int M, bool kFull>
+__global__ void __launch_bounds__(kTpThr, (tile_ctas<float, M>()))
     k_batch(float2 *__restrict__ scratch, const BCirc *__restrict__ circs, const BPass *__restrict__ passes,
-            const StOp<float> *__restrict__ ops, const BItem *__restrict__ items, int64_t nitems, BCtl *ctl, int *done,
+            const uint4 *__restrict__ progs, const BItem *__restrict__ items, int64_t nitems, BCtl *ctl, int *done,
             int *finished, double *__restrict__ partial, double *__restrict__ out)
 {
-    constexpr int RB = M - kThrBits, RA = 1 << RB;
+    constexpr int RB = M - kTpThrBits, RA = 1 << RB;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float *sm = reinterpret_cast<float *>(smem_raw);
+    uint4 *sp = reinterpret_cast<uint4 *>(smem_raw + (size_t)tile_slots<M, RB, 2>() * sizeof(float2));
     __shared__ long long cur;
     __shared__ int stop;
-    __shared__ double red[kThr / 32];
+    __shared__ double red[kTpThr / 32];
     __shared__ int last;
     const int tid = threadIdx.x;
 
@@ -127,84 +128,50 @@ __global__ void __launch_bounds__(kThr, M <= 12 ? 3 : 2)
             if (stop) break;
         }
 
-        // tile base and I/O offsets (layout 0).  They are formed again after
-        // the gate sequence from inputs the compiler cannot prove equal
-        // instead of being held live across it (which spilled at two CTAs
-        // per SM), as in the staged kernel.
-        uint64_t base = 0;
-        for (int i = 0; i < ps.geo.n_outer; ++i) base |= ((uint64_t)(it.tile >> i) & 1ull) << ps.geo.outer_pos[i];
-        uint64_t toff, roff[RB];
-        auto io_offsets = [&](const TileGeom &geo, int t, uint64_t b0) {
-            toff = b0;
-#pragma unroll
-            for (int i = 0; i < kThrBits; ++i) {
-                const int b = thr_local(M, RB, 2, 0, i);
-                const uint64_t g = (b < kLow) ? (1ull << b) : (1ull << geo.hpos[b - kLow]);
-                if ((t >> i) & 1) toff |= g;
-            }
-#pragma unroll
-            for (int j = 0; j < RB; ++j) {
-                const int b = reg_local(M, RB, 2, 0, j);
-                roff[j] = (b < kLow) ? (1ull << b) : (1ull << geo.hpos[b - kLow]);
-            }
-        };
-        io_offsets(ps.geo, tid, base);
+        const uint4 *prog = progs + ps.prog0;
+        const int nunits = ps.nunits;
+        prog_stage(prog, nunits, tid, sp);
+        uint64_t base = tile_base(ps.geo, (uint32_t)it.tile);
         float *st = reinterpret_cast<float *>(scratch + c.state0);
 
-        Regs<float, RA> v;
+        Amps<float, RA> v;
         if (it.pass == 0) {
             // |0...0>: amplitude 0 sits in register 0 of thread 0 of tile 0
 #pragma unroll
-            for (int p = 0; p < RA / 2; ++p) v.set2(p, 0.f, 0.f, 0.f, 0.f);
-            if (base == 0 && tid == 0) v.setr(0, 1.f);
+            for (int p = 0; p < RA / 2; ++p) v.r[p] = v.i[p] = 0ull;
+            if (it.tile == 0 && tid == 0) v.set(0, 1.f, 0.f);
         } else {
-#pragma unroll
-            for (int k = 0; k < RA; k += 2) {
-                uint64_t g = toff;
-#pragma unroll
-                for (int j = 1; j < RB; ++j)
-                    if ((k >> j) & 1) g |= roff[j];
-                const float4 t = __ldcg(reinterpret_cast<const float4 *>(st + 2 * g));
-                v.set2(k >> 1, t.x, t.y, t.z, t.w);
-            }
+            tile_load<M, RB, 2, true>(ps.start_layout, v, st, ps.geo, tid, base);
         }
-
-        apply_ops<float, M>(v, ops + ps.op0, ps.nops, base, tid, sm,
-                            reinterpret_cast<StOp<float> *>(smem_raw + ((size_t)1 << M) * 2 * sizeof(float)));
-        {
-            int t2 = tid;
-            uint64_t b2 = base;
-            const BPass *pp = passes + (c.pass0 + it.pass);
-            asm volatile("" : "+r"(t2), "+l"(b2), "+l"(pp));
-            io_offsets(pp->geo, t2, b2);
-        }
+        __syncthreads();
+        run_program<float, M, kFull>(v, prog, nunits, (uint32_t)it.tile, tid, sm, sp);
 
         if (it.pass + 1 < c.npass) {
-#pragma unroll
-            for (int k = 0; k < RA; k += 2) {
-                uint64_t g = toff;
-#pragma unroll
-                for (int j = 1; j < RB; ++j)
-                    if ((k >> j) & 1) g |= roff[j];
-                __stcg(reinterpret_cast<float4 *>(st + 2 * g),
-                       make_float4(v.getr(k), v.geti(k), v.getr(k + 1), v.geti(k + 1)));
-            }
+            // addresses formed again instead of being held live across the program
+            int t2 = tid;
+            const BPass *pp = passes + (c.pass0 + it.pass);
+            asm volatile("" : "+r"(t2), "+l"(base), "+l"(pp));
+            tile_store<M, RB, 2, true>(pp->end_layout, v, st, pp->geo, t2, base, pp->flip);
             __syncthreads();
             if (tid == 0) {
                 __threadfence();
                 atomicAdd(done + c.pass0 + it.pass, 1);
             }
         } else {
-            // <sum Z> over this tile: |a_x|^2 (n - 2 popcount x), FP64
+            // <sum Z> over this tile: |a_x|^2 (n - 2 popcount x), FP64.  Every
+            // thread and register bit is one qubit, so the popcount of x is
+            // that of the outer bits, the thread and the register (exchanged
+            // labels included), whatever the layout.
+            const BPass *pp = passes + (c.pass0 + it.pass);
+            const uint64_t flip = pp->flip;
+            uint32_t fthr = 0, freg = 0;
+            flip_bits<M, RB, 2>(pp->end_layout, pp->geo, flip, &fthr, &freg);
+            const int w0 = c.n - 2 * (__popcll(base) + __popc((uint32_t)tid ^ fthr));
             double acc = 0.0;
 #pragma unroll
             for (int k = 0; k < RA; ++k) {
-                uint64_t g = toff;
-#pragma unroll
-                for (int j = 0; j < RB; ++j)
-                    if ((k >> j) & 1) g |= roff[j];
-                const double re = v.getr(k), im = v.geti(k);
-                acc += (re * re + im * im) * (double)(c.n - 2 * __popcll(g));
+                const double re = v.re(k), im = v.im(k);
+                acc += (re * re + im * im) * (double)(w0 - 2 * __popc((uint32_t)k ^ freg));
             }
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
@@ -212,7 +179,7 @@ __global__ void __launch_bounds__(kThr, M <= 12 ? 3 : 2)
             __syncthreads();
             if (tid == 0) {
                 double s = 0.0;
-                for (int w = 0; w < kThr / 32; ++w) s += red[w];
+                for (int w = 0; w < kTpThr / 32; ++w) s += red[w];
                 if (single) {
                     out[it.circ] = s;
                     last = 0;
@@ -283,7 +250,7 @@ struct qsim_batch {
     void *dev = nullptr;              // one allocation for everything
     BCirc *circs = nullptr;
     BPass *passes = nullptr;
-    StOp<float> *ops = nullptr;
+    uint4 *progs = nullptr;
     BItem *items = nullptr;
     BCtl *ctl = nullptr;
     int *done = nullptr, *finished = nullptr;
@@ -306,12 +273,12 @@ static void batch_free(qsim_batch *b)
 
 namespace {
 
-template <int M>
-const void *batch_kernel() { return (const void *)k_batch<M>; }
-
-const void *batch_kernel_for(int M)
+// full: some program holds other operations than groups
+const void *batch_kernel_for(int M, bool full)
 {
-    return M == 11 ? batch_kernel<11>() : M == 12 ? batch_kernel<12>() : batch_kernel<13>();
+    if (M == 11) return full ? (const void *)k_batch<11, true> : (const void *)k_batch<11, false>;
+    if (M == 12) return full ? (const void *)k_batch<12, true> : (const void *)k_batch<12, false>;
+    return full ? (const void *)k_batch<13, true> : (const void *)k_batch<13, false>;
 }
 
 }  // namespace
@@ -342,30 +309,33 @@ extern "C" int sim_batch_create_opts(int count, const int32_t *n_qubits, const i
 
     std::vector<BCirc> circs(count);
     std::vector<BPass> passes;
-    std::vector<StOp<float>> ops;
+    std::vector<uint32_t> words;
+    int64_t nops = 0;
+    bool full = false;
     int64_t state_amps = 0, parts = 0;
     double alg_flops = 0, alg_scratch = 0;
     for (int c = 0; c < count; ++c) {
         const int n = n_qubits[c];
         std::vector<SGate> g;
-        lower_gates(gates + gate_offsets[c], (size_t)(gate_offsets[c + 1] - gate_offsets[c]), &g);
+        lower_renamed(gates + gate_offsets[c], (size_t)(gate_offsets[c + 1] - gate_offsets[c]), n, &g);
+        // <sum Z> does not depend on where the qubits end up
+        while (!g.empty() && g.back().op == OP_SWAP) g.pop_back();
         for (const SGate &sg : g) alg_flops += sgate_flops(sg, n);
         merge_single_qubit(&g);
         const int nplan = std::max(n, M);           // below M qubits: phantom qubits that stay |0>
-        std::vector<Pass> ps = form_passes(g, nplan, M);
-        if (ps.empty()) {
-            Pass empty_pass;
-            for (int q = kLow; q < M; ++q) empty_pass.high.push_back(q);
-            ps.push_back(empty_pass);
+        std::vector<Program> progs = compile_passes<float>(g, nplan, M, 2, true);
+        if (progs.empty()) {                        // no gates: one pass that does nothing
+            Program none;
+            for (int q = kLow; q < M; ++q) none.pass.high.push_back(q);
+            pack_program<float>(none.tp, &none.words);
+            progs.push_back(none);
         }
         // scratch traffic the plan must make: every pass but the first reads
         // the state, every pass but the last writes it (8 B per amplitude)
-        if (ps.size() > 1) alg_scratch += 2.0 * (double)(ps.size() - 1) * std::ldexp(8.0, nplan);
-        PlanBuilder<float> pb{nplan, M, M - kThrBits, 2, {}, {}, 0};
-        pb.allow_ramps = false;   // the batched kernel runs the tile engine without ramps
+        if (progs.size() > 1) alg_scratch += 2.0 * (double)(progs.size() - 1) * std::ldexp(8.0, nplan);
         BCirc bc{};
         bc.n = n;
-        bc.npass = (int)ps.size();
+        bc.npass = (int)progs.size();
         bc.ntiles = 1 << (nplan - M);
         bc.pass0 = (int64_t)passes.size();
         bc.part0 = parts;
@@ -375,23 +345,22 @@ extern "C" int sim_batch_create_opts(int count, const int32_t *n_qubits, const i
             state_amps += (int64_t)1 << nplan;
         }
         parts += bc.ntiles;
-        for (const Pass &p : ps) {
+        for (const Program &p : progs) {
             BPass bp;
             memset(&bp, 0, sizeof bp);
-            bp.op0 = (int64_t)(ops.size() + pb.ops.size());
-            bp.nops = pb.schedule(p, g);
+            bp.prog0 = (int64_t)(words.size() / 4);
+            bp.nunits = (int)(p.words.size() / 4);
             bp.need = bc.ntiles;
-            uint64_t q = (1ull << kLow) - 1ull;
-            for (size_t i = 0; i < p.high.size(); ++i) {
-                bp.geo.hpos[i] = p.high[i];
-                q |= 1ull << p.high[i];
-            }
-            for (int b2 = 0; b2 < nplan; ++b2)
-                if (!((q >> b2) & 1)) bp.geo.outer_pos[bp.geo.n_outer++] = b2;
+            bp.start_layout = p.tp.start_layout;
+            bp.end_layout = p.tp.end_layout;
+            bp.flip = p.tp.flip;
+            bp.geo = tile_geom(p.pass, nplan);
+            words.insert(words.end(), p.words.begin(), p.words.end());
+            nops += (int64_t)p.tp.ops.size();
+            full = full || !p.tp.groups_only();
             passes.push_back(bp);
         }
         if (inject_stall && c == 0 && bc.npass > 1) passes[bc.pass0 + 1].need = bc.ntiles + 1;
-        ops.insert(ops.end(), pb.ops.begin(), pb.ops.end());
         circs[c] = bc;
     }
     // queue: pass index major, circuits by descending work, tiles ascending
@@ -415,7 +384,7 @@ extern "C" int sim_batch_create_opts(int count, const int32_t *n_qubits, const i
     b->alg_scratch_bytes = alg_scratch;
     b->nitems = (int64_t)items.size();
     b->npasses = (int64_t)passes.size();
-    b->nops = (int64_t)ops.size();
+    b->nops = nops;
     int rc = SIM_OK;
     do {
         if (stream) {
@@ -431,7 +400,7 @@ extern "C" int sim_batch_create_opts(int count, const int32_t *n_qubits, const i
         size_t off = 0;
         const size_t o_c = off; off += al(sizeof(BCirc) * count);
         const size_t o_p = off; off += al(sizeof(BPass) * passes.size());
-        const size_t o_o = off; off += al(sizeof(StOp<float>) * std::max<size_t>(ops.size(), 1));
+        const size_t o_o = off; off += al(words.size() * 4);
         const size_t o_i = off; off += al(sizeof(BItem) * items.size());
         const size_t o_ctl = off; off += al(sizeof(BCtl));
         const size_t o_d = off; off += al(sizeof(int) * passes.size());
@@ -448,7 +417,7 @@ extern "C" int sim_batch_create_opts(int count, const int32_t *n_qubits, const i
         char *d = (char *)b->dev;
         b->circs = (BCirc *)(d + o_c);
         b->passes = (BPass *)(d + o_p);
-        b->ops = (StOp<float> *)(d + o_o);
+        b->progs = (uint4 *)(d + o_o);
         b->items = (BItem *)(d + o_i);
         b->ctl = (BCtl *)(d + o_ctl);
         b->done = (int *)(d + o_d);
@@ -458,18 +427,18 @@ extern "C" int sim_batch_create_opts(int count, const int32_t *n_qubits, const i
         b->scratch = (float2 *)(d + o_s);
         if (cudaMemcpy(b->circs, circs.data(), sizeof(BCirc) * count, cudaMemcpyHostToDevice) != cudaSuccess ||
             cudaMemcpy(b->passes, passes.data(), sizeof(BPass) * passes.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
-            (!ops.empty() && cudaMemcpy(b->ops, ops.data(), sizeof(StOp<float>) * ops.size(), cudaMemcpyHostToDevice) != cudaSuccess) ||
+            cudaMemcpy(b->progs, words.data(), words.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess ||
             cudaMemcpy(b->items, items.data(), sizeof(BItem) * items.size(), cudaMemcpyHostToDevice) != cudaSuccess) {
             rc = cuda_fail(cudaGetLastError(), "sim_batch_create: upload");
             break;
         }
-        const void *kern = batch_kernel_for(M);
-        const size_t smem = ((size_t)1 << M) * 2 * sizeof(float) + op_stage_bytes<float>();
+        const void *kern = batch_kernel_for(M, full);
+        const size_t smem = M == 11 ? tile_smem_bytes<float, 11>() : M == 12 ? tile_smem_bytes<float, 12>() : tile_smem_bytes<float, 13>();
         if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
             rc = cuda_fail(cudaGetLastError(), "batch smem attribute");
             break;
         }
-        // up to two (13-qubit tiles) or three CTAs per SM
+        // as many CTAs per SM as the tiles' shared memory allows
         if (cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
                                  (int)cudaSharedmemCarveoutMaxShared) != cudaSuccess) {
             rc = cuda_fail(cudaGetLastError(), "batch carveout attribute");
@@ -478,7 +447,7 @@ extern "C" int sim_batch_create_opts(int count, const int32_t *n_qubits, const i
         int dev = 0, sms = 0, per_sm = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThr, smem) != cudaSuccess || per_sm < 1) {
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kTpThr, smem) != cudaSuccess || per_sm < 1) {
             rc = fail(SIM_ECUDA, "sim_batch_create: persistent kernel does not fit on an SM");
             break;
         }
@@ -502,15 +471,9 @@ extern "C" int sim_batch_create_opts(int count, const int32_t *n_qubits, const i
         }
         cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
         k_batch_reset<<<64, 256, 0, cs>>>(b->ctl, b->done, b->npasses, b->finished, count);
-        if (M == 11)
-            k_batch<11><<<b->grid, kThr, smem, cs>>>(b->scratch, b->circs, b->passes, b->ops, b->items, b->nitems,
-                                                    b->ctl, b->done, b->finished, b->partial, b->out);
-        else if (M == 12)
-            k_batch<12><<<b->grid, kThr, smem, cs>>>(b->scratch, b->circs, b->passes, b->ops, b->items, b->nitems,
-                                                    b->ctl, b->done, b->finished, b->partial, b->out);
-        else
-            k_batch<13><<<b->grid, kThr, smem, cs>>>(b->scratch, b->circs, b->passes, b->ops, b->items, b->nitems,
-                                                    b->ctl, b->done, b->finished, b->partial, b->out);
+        void *args[] = {&b->scratch, &b->circs, &b->passes, &b->progs, &b->items, &b->nitems, &b->ctl, &b->done,
+                        &b->finished, &b->partial, &b->out};
+        cudaLaunchKernel(kern, dim3((unsigned)b->grid), dim3(kTpThr), args, smem, cs);
         cudaError_t ce = cudaStreamEndCapture(cs, &b->graph);
         cudaStreamDestroy(cs);
         if (ce != cudaSuccess) {

@@ -174,15 +174,15 @@ bool sample_observe_fused(const qsim_state *s);
 // matrix on one target with a set of control qubits.  SWAP is lowered to
 // three CNOT-type moves; identity gates are dropped.
 struct SGate {
-    int op;              // GateOp (no OP_SWAP / OP_IDENTITY here)
+    int op;              // GateOp (no OP_IDENTITY; OP_SWAP, without controls, from lower_renamed only)
     int target;
     uint64_t ctrl;       // control qubits
     double m[8];
     int orig;            // index of the circuit gate it comes from (OP_SUPER: index of its 4 x 4 matrix)
-    int target2 = -1;    // OP_SUPER: the second qubit (above target)
+    int target2 = -1;    // OP_SUPER: the second qubit (above target); OP_SWAP: the partner
     uint64_t xq() const
     {
-        if (op == OP_SUPER) return (1ull << target) | (1ull << target2);
+        if (op == OP_SUPER || op == OP_SWAP) return (1ull << target) | (1ull << target2);
         return (op == OP_DENSE || op == OP_ANTIDIAG || op == OP_XPERM) ? (1ull << target) : 0ull;
     }
     uint64_t dq() const { return ctrl | ((op == OP_DIAG || op == OP_DIAG_HI) ? (1ull << target) : 0ull); }
@@ -191,6 +191,10 @@ struct SGate {
 // true when the two gates commute: every shared qubit is acted on diagonally by both
 bool commute(const SGate &a, const SGate &b);
 void lower_gates(const sim_gate *gates, size_t n_gates, std::vector<SGate> *out);
+// the same, but SWAP gates without controls rename the qubits of every later
+// gate instead of moving amplitudes; what is left of the renaming at the end
+// comes as OP_SWAP gates
+void lower_renamed(const sim_gate *gates, size_t n_gates, int n, std::vector<SGate> *out);
 
 // one lowered gate (up to 3 controls) as its own per-gate launch
 int launch_sgate(qsim_state *s, const SGate &g);
@@ -202,6 +206,14 @@ int apply_circuit_fused(qsim_state *s, const sim_gate *gates, size_t n_gates, co
 // (a density matrix's channels; sup = their 4 x 4 matrices, 32 doubles each,
 // row-major (re, im), indexed by SGate::orig)
 int apply_sgates_fused(qsim_state *s, const std::vector<SGate> &g, const double *sup, int k);
+// register-tile passes over lowered gates (lower_renamed), with the tile size
+// tile_cost assumes; and their predicted time, in microseconds on 2^26
+// amplitudes (host only)
+int run_tiles(qsim_state *s, const std::vector<SGate> &g);
+double tile_cost(const std::vector<SGate> &g, int n, int dtype);
+// registers from this size on: the fused plan with the largest blocks takes
+// tile passes for the stretches they are predicted to be faster on
+bool fused_mixes(int n, int dtype, int k);
 int apply_circuit_learned(qsim_state *s, const sim_gate *gates, size_t n_gates, const sim_plan_opts &o);
 int plan_features(int n, int dtype, const sim_gate *gates, size_t n_gates, int v, float *out);
 // the learned plan's variant per window for a complex64 register with a cost
@@ -218,6 +230,9 @@ int describe_staged(int n, int dtype, const sim_gate *gates, size_t n_gates, int
                     int64_t *ops, int64_t *layout_changes, int32_t *order, size_t order_cap, size_t *order_len);
 int encode_staged(int n, int dtype, const sim_gate *gates, size_t n_gates, int tile_qubits, sim_tile_op *ops,
                   size_t ops_cap, int32_t *info, size_t info_cap, size_t *n_ops, size_t *n_passes);
+
+int export_tile_programs(int n, int dtype, const sim_gate *gates, size_t n_gates, int tile_qubits, uint32_t *words,
+                         size_t words_cap, int32_t *info, size_t info_cap, size_t *n_words, size_t *n_passes);
 
 // f(0) .. f(count - 1) on up to 16 host threads: the calling thread and a
 // persistent pool (pool.cu).  Serial for one index, inside a pool thread, or

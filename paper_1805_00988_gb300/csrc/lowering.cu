@@ -1,4 +1,5 @@
 // lowering.cu -- circuit gates to the planners' gate form.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <vector>
@@ -14,29 +15,59 @@ bool commute(const SGate &a, const SGate &b)
 }
 
 // SWAP(a, b) with controls c = CNOT(b -> a) . X(target b; controls c + a) . CNOT(b -> a)
-void lower_gates(const sim_gate *gates, size_t n_gates, std::vector<SGate> *out)
+static void lower_one(const sim_gate &gate, size_t k, const int *at, std::vector<SGate> *out)
 {
     static const double X[8] = {0, 0, 1, 0, 1, 0, 0, 0};
-    for (size_t k = 0; k < n_gates; ++k) {
-        const PairGate p = make_pair_gate(gates[k]);
-        uint64_t cm = 0;
-        for (int c = 0; c < p.nctrl; ++c) cm |= 1ull << p.ctrl[c];
-        if (p.op == OP_IDENTITY) continue;
-        if (p.op == OP_SWAP) {
-            const int a = p.target, b = p.target2;
-            SGate g1{OP_XPERM, a, 1ull << b, {}, (int)k};
-            SGate g2{OP_XPERM, b, cm | (1ull << a), {}, (int)k};
-            memcpy(g1.m, X, sizeof X);
-            memcpy(g2.m, X, sizeof X);
-            out->push_back(g1);
-            out->push_back(g2);
-            out->push_back(g1);
-            continue;
-        }
-        SGate g{p.op, p.target, cm, {}, (int)k};
-        memcpy(g.m, p.m, sizeof g.m);
-        out->push_back(g);
+    const PairGate p = make_pair_gate(gate);
+    uint64_t cm = 0;
+    for (int c = 0; c < p.nctrl; ++c) cm |= 1ull << at[p.ctrl[c]];
+    if (p.op == OP_IDENTITY) return;
+    if (p.op == OP_SWAP) {
+        const int a = at[p.target], b = at[p.target2];
+        SGate g1{OP_XPERM, a, 1ull << b, {}, (int)k};
+        SGate g2{OP_XPERM, b, cm | (1ull << a), {}, (int)k};
+        memcpy(g1.m, X, sizeof X);
+        memcpy(g2.m, X, sizeof X);
+        out->push_back(g1);
+        out->push_back(g2);
+        out->push_back(g1);
+        return;
     }
+    SGate g{p.op, at[p.target], cm, {}, (int)k};
+    memcpy(g.m, p.m, sizeof g.m);
+    out->push_back(g);
+}
+
+void lower_gates(const sim_gate *gates, size_t n_gates, std::vector<SGate> *out)
+{
+    int same[64];
+    for (int q = 0; q < 64; ++q) same[q] = q;
+    for (size_t k = 0; k < n_gates; ++k) lower_one(gates[k], k, same, out);
+}
+
+void lower_renamed(const sim_gate *gates, size_t n_gates, int n, std::vector<SGate> *out)
+{
+    int at[64];                    // where the circuit's qubit q lives
+    for (int q = 0; q < 64; ++q) at[q] = q;
+    for (size_t k = 0; k < n_gates; ++k) {
+        if (gates[k].kind == SIM_GATE_SWAP && gates[k].n_controls == 0) std::swap(at[gates[k].target], at[gates[k].target2]);
+        else lower_one(gates[k], k, at, out);
+    }
+    // bring qubit q back to place q, one exchange of places after the other
+    // (around the lowest place of each cycle, which most tiles hold)
+    for (int q = 0; q < n; ++q)
+        while (at[q] != q) {
+            const int p = at[q];              // place q holds another qubit; swap places q and p
+            SGate g{OP_SWAP, std::min(p, q), 0, {}, -1};
+            g.target2 = std::max(p, q);
+            out->push_back(g);
+            for (int r = 0; r < n; ++r)
+                if (at[r] == q && r != q) {
+                    at[r] = p;
+                    break;
+                }
+            at[q] = q;
+        }
 }
 
 double sgate_flops(const SGate &g, int n)

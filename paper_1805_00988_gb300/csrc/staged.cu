@@ -10,194 +10,144 @@
 // gates (Z, S, T, P, RZ, CZ, CP, ...) and controls never need their qubit in
 // Q: outside Q the bit is constant over the tile.
 //
-// Inside a CTA the tile lives in registers: with 256 threads each thread holds
-// 2^(M-8) amplitudes.  A register layout assigns the tile's local bits to
+// Inside a CTA the tile lives in registers: with 128 threads each thread holds
+// 2^(M-7) amplitudes.  A register layout assigns the tile's local bits to
 // register bits and thread bits; a gate whose target is a register bit is
 // applied by each thread alone.  Layouts change through shared memory (one
-// store + one load of the tile, XOR-swizzled so every layout is free of bank
-// conflicts).  The host planner (below) forms the passes, orders the gates of
-// a pass to need few layout changes, and encodes each gate as register /
-// thread / tile masks for the layout current at that point.
+// store + one load of the tile, padded so the layouts are free of bank
+// conflicts).  The host planner forms the passes (tile.cuh); the gates of a
+// pass are ordered and compiled into a tile program (tileprog.cuh), which the
+// kernel below runs.
 #include <algorithm>
 #include <cstring>
 #include <vector>
 
-#include "tile.cuh"
+#include "tileprog.cuh"
 
 namespace qsim {
 
 namespace {
 
-// complex64 tiles of up to 12 qubits hold 16 amplitudes a thread and fit 80
-// registers: three CTAs per SM; 13-qubit and complex128 tiles two.  kRamp:
-// the variant that also runs SK_RAMP ops, launched for the passes that have
-// them.
-template <typename R, int M, bool kRamp>
-__global__ void __launch_bounds__(kThr, (sizeof(R) == 4 && M <= 12 ? 3 : 2))
-k_staged(R *__restrict__ st, const StOp<R> *__restrict__ ops, int nops,
-                                                   TileGeom geo)
+template <typename R, int M, bool kFull>
+__global__ void __launch_bounds__(kTpThr, (tile_ctas<R, M>()))
+    k_staged(R *__restrict__ st, const uint4 *__restrict__ prog, int nunits, TileGeom geo, int start_layout,
+             int end_layout, uint64_t flip)
 {
     constexpr int VEC = (sizeof(R) == 4) ? 2 : 1;
-    constexpr int RB = M - kThrBits;
-    constexpr int RA = 1 << RB;
+    constexpr int RB = M - kTpThrBits;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     R *sm = reinterpret_cast<R *>(smem_raw);
+    uint4 *sp = reinterpret_cast<uint4 *>(smem_raw + (size_t)tile_slots<M, RB, VEC>() * 2 * sizeof(R));
     const int tid = threadIdx.x;
+    const uint32_t tile = blockIdx.x;
 
-    const uint64_t tile = (uint64_t)blockIdx.x;
-    uint64_t base = 0;
-    for (int i = 0; i < geo.n_outer; ++i) base |= ((tile >> i) & 1ull) << geo.outer_pos[i];
-
-    // global offsets in the I/O layout: the thread's offset and one per
-    // register bit.  They are formed again for the store (from inputs the
-    // compiler cannot prove equal) instead of being held live across the
-    // gate sequence, which would spill at two CTAs per SM.
-    uint64_t toff, roff[RB];
-    auto io_offsets = [&](int t, uint64_t b0) {
-        toff = b0;
-#pragma unroll
-        for (int i = 0; i < kThrBits; ++i) {
-            const int b = thr_local(M, RB, VEC, 0, i);
-            const uint64_t g = (b < kLow) ? (1ull << b) : (1ull << geo.hpos[b - kLow]);
-            if ((t >> i) & 1) toff |= g;
-        }
-#pragma unroll
-        for (int j = 0; j < RB; ++j) {
-            const int b = reg_local(M, RB, VEC, 0, j);
-            roff[j] = (b < kLow) ? (1ull << b) : (1ull << geo.hpos[b - kLow]);
-        }
-    };
-    io_offsets(tid, base);
-
-    Regs<R, RA> v;
-    if constexpr (VEC == 2) {
-#pragma unroll
-        for (int k = 0; k < RA; k += 2) {
-            uint64_t g = toff;
-#pragma unroll
-            for (int j = 1; j < RB; ++j)
-                if ((k >> j) & 1) g |= roff[j];
-            const float4 t = *reinterpret_cast<const float4 *>(st + 2 * g);
-            v.set2(k >> 1, t.x, t.y, t.z, t.w);
-        }
-    } else {
-#pragma unroll
-        for (int k = 0; k < RA; ++k) {
-            uint64_t g = toff;
-#pragma unroll
-            for (int j = 0; j < RB; ++j)
-                if ((k >> j) & 1) g |= roff[j];
-            const double2 t = *reinterpret_cast<const double2 *>(st + 2 * g);
-            v.setr(k, (R)t.x);
-            v.seti(k, (R)t.y);
-        }
-    }
-
-    apply_ops<R, M, kRamp>(v, ops, nops, base, tid, sm,
-                    reinterpret_cast<StOp<R> *>(smem_raw + ((size_t)1 << M) * 2 * sizeof(R)));
-    {
-        int t2 = tid;
-        uint64_t b2 = base;
-        asm volatile("" : "+r"(t2), "+l"(b2));
-        io_offsets(t2, b2);
-    }
-    // the planner always ends a pass in layout 0
-    if constexpr (VEC == 2) {
-#pragma unroll
-        for (int k = 0; k < RA; k += 2) {
-            uint64_t g = toff;
-#pragma unroll
-            for (int j = 1; j < RB; ++j)
-                if ((k >> j) & 1) g |= roff[j];
-            *reinterpret_cast<float4 *>(st + 2 * g) = make_float4(v.getr(k), v.geti(k), v.getr(k + 1), v.geti(k + 1));
-        }
-    } else {
-#pragma unroll
-        for (int k = 0; k < RA; ++k) {
-            uint64_t g = toff;
-#pragma unroll
-            for (int j = 0; j < RB; ++j)
-                if ((k >> j) & 1) g |= roff[j];
-            *reinterpret_cast<double2 *>(st + 2 * g) = make_double2((double)v.getr(k), (double)v.geti(k));
-        }
-    }
+    prog_stage(prog, nunits, tid, sp);
+    uint64_t base = tile_base(geo, tile);
+    Amps<R, (1 << RB)> v;
+    tile_load<M, RB, VEC, false>(start_layout, v, st, geo, tid, base);
+    __syncthreads();
+    run_program<R, M, kFull>(v, prog, nunits, tile, tid, sm, sp);
+    // addresses are formed again from inputs the compiler cannot prove equal,
+    // instead of being held live across the program
+    int t2 = tid;
+    asm volatile("" : "+r"(t2), "+l"(base));
+    tile_store<M, RB, VEC, false>(end_layout, v, st, geo, t2, base, flip);
 }
 
-template <typename R, int M, bool kRamp>
-int launch_staged_v(qsim_state *s, const StOp<R> *dops, int nops, const TileGeom &geo, double flops)
+template <typename R, int M, bool kFull>
+int launch_staged_v(qsim_state *s, const uint4 *prog, int nunits, const TileGeom &geo, const TilePass &tp, double flops)
 {
-    const size_t smem = ((size_t)1 << M) * 2 * sizeof(R) + op_stage_bytes<R>();
+    const size_t smem = tile_smem_bytes<R, M>();
     // set on every launch: the attribute belongs to the current device's
     // context, and the call costs a microsecond against a multi-ms pass
-    QSIM_CUDA(cudaFuncSetAttribute(k_staged<R, M, kRamp>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    QSIM_CUDA(cudaFuncSetAttribute(k_staged<R, M, kFull>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     const uint64_t tiles = 1ull << (s->n - M);
     launch_begin(s, KC_STAGED, 2.0 * (double)s->bytes, flops);
-    k_staged<R, M, kRamp><<<(unsigned)tiles, kThr, smem, s->stream>>>((R *)s->amps, dops, nops, geo);
+    k_staged<R, M, kFull><<<(unsigned)tiles, kTpThr, smem, s->stream>>>((R *)s->amps, prog, nunits, geo,
+                                                                        tp.start_layout, tp.end_layout, tp.flip);
     return launch_end(s, "staged pass");
 }
 
 template <typename R, int M>
-int launch_staged(qsim_state *s, const StOp<R> *dops, int nops, const TileGeom &geo, double flops, bool ramp)
+int launch_staged(qsim_state *s, const uint4 *prog, int nunits, const TileGeom &geo, const TilePass &tp, double flops)
 {
-    return ramp ? launch_staged_v<R, M, true>(s, dops, nops, geo, flops)
-                : launch_staged_v<R, M, false>(s, dops, nops, geo, flops);
+    // complex128 passes are bound by the FP64 pipe: one variant is enough
+    if (sizeof(R) == 4 && tp.groups_only()) {
+        if constexpr (sizeof(R) == 4) return launch_staged_v<R, M, false>(s, prog, nunits, geo, tp, flops);
+    }
+    return launch_staged_v<R, M, true>(s, prog, nunits, geo, tp, flops);
+}
+
+// Programs are planned, copied and launched one pass at a time, so the host
+// plans the next pass while the GPU runs this one (a 20-qubit random circuit
+// spent 0.45 ms planning before 0.27 ms of kernels).  They go through one
+// pinned buffer, each at its own place; when it is full the stream is waited
+// for and the buffer starts again.
+constexpr size_t kProgBuffer = (size_t)1 << 18;
+
+template <typename R, int M>
+int run_staged(qsim_state *s, const std::vector<SGate> &g)
+{
+    const int VEC = sizeof(R) == 4 ? 2 : 1;
+    TilePlanner<R> plan(g, s->n, M, VEC);
+    Program p;
+    size_t off = 0;
+    int rc = SIM_OK;
+    while (rc == SIM_OK && plan.next(&p)) {
+        const size_t bytes = p.words.size() * 4;
+        if (off + bytes > s->host_ops_bytes || off + bytes > s->dev_ops_bytes) {
+            if (off) QSIM_CUDA(cudaStreamSynchronize(s->stream));
+            off = 0;
+            const size_t need = std::max(kProgBuffer, 2 * bytes);
+            if ((rc = ensure_host_pinned(&s->host_ops, &s->host_ops_bytes, need))) break;
+            if ((rc = ensure_device(s, &s->dev_ops, &s->dev_ops_bytes, need))) break;
+        }
+        memcpy((char *)s->host_ops + off, p.words.data(), bytes);
+        uint4 *prog = (uint4 *)((char *)s->dev_ops + off);
+        if (cudaMemcpyAsync(prog, (char *)s->host_ops + off, bytes, cudaMemcpyHostToDevice, s->stream) != cudaSuccess) {
+            rc = cuda_fail(cudaGetLastError(), "tile program upload");
+            break;
+        }
+        double f = 0.0;
+        for (int m : p.members) f += sgate_flops(g[(size_t)m], s->n);
+        rc = launch_staged<R, M>(s, prog, (int)(p.words.size() / 4), tile_geom(p.pass, s->n), p.tp, f);
+        off += (bytes + 255) & ~(size_t)255;
+    }
+    // the pinned buffer is reused by the next call: wait for the copies
+    const cudaError_t e = cudaStreamSynchronize(s->stream);
+    if (rc == SIM_OK && e != cudaSuccess) rc = cuda_fail(e, "staged plan");
+    return rc;
 }
 
 template <typename R>
 int run_staged(qsim_state *s, const std::vector<SGate> &g, int M)
 {
-    const int VEC = sizeof(R) == 4 ? 2 : 1;
-    std::vector<Pass> passes = form_passes(g, s->n, M);
-    PlanBuilder<R> pb{s->n, M, M - kThrBits, VEC, {}, {}, 0};
-    std::vector<int> counts;
-    std::vector<double> pflops;
-    std::vector<char> ramp;
-    for (const Pass &ps : passes) {
-        const size_t first = pb.ops.size();
-        counts.push_back(pb.schedule(ps, g));
-        bool r = false;
-        for (size_t k = first; k < pb.ops.size() && !r; ++k) r = pb.ops[k].kind == SK_RAMP;
-        ramp.push_back(r);
-        double f = 0.0;
-        for (int m : ps.members) f += sgate_flops(g[m], s->n);
-        pflops.push_back(f);
-    }
-    const size_t bytes = pb.ops.size() * sizeof(StOp<R>);
-    if (int rc = ensure_host_pinned(&s->host_ops, &s->host_ops_bytes, bytes)) return rc;
-    if (int rc = ensure_device(s, &s->dev_ops, &s->dev_ops_bytes, bytes)) return rc;
-    memcpy(s->host_ops, pb.ops.data(), bytes);
-    QSIM_CUDA(cudaMemcpyAsync(s->dev_ops, s->host_ops, bytes, cudaMemcpyHostToDevice, s->stream));
-    const StOp<R> *dops = (const StOp<R> *)s->dev_ops;
-    size_t off = 0;
-    for (size_t p = 0; p < passes.size(); ++p) {
-        TileGeom geo;
-        memset(&geo, 0, sizeof geo);
-        uint64_t q = (1ull << kLow) - 1ull;
-        for (size_t i = 0; i < passes[p].high.size(); ++i) {
-            geo.hpos[i] = passes[p].high[i];
-            q |= 1ull << passes[p].high[i];
-        }
-        for (int b = 0; b < s->n; ++b)
-            if (!((q >> b) & 1)) geo.outer_pos[geo.n_outer++] = b;
-        int rc;
-        switch (M) {
-        case 11: rc = launch_staged<R, 11>(s, dops + off, counts[p], geo, pflops[p], ramp[p]); break;
-        case 12: rc = launch_staged<R, 12>(s, dops + off, counts[p], geo, pflops[p], ramp[p]); break;
-        case 13:
-            if constexpr (sizeof(R) == 4) rc = launch_staged<R, 13>(s, dops + off, counts[p], geo, pflops[p], ramp[p]);
-            else rc = fail(SIM_EINVAL, "staged: complex128 tiles are at most 12 qubits");
-            break;
-        default: rc = fail(SIM_EINVAL, "staged: unsupported tile size");
-        }
-        if (rc) return rc;
-        off += counts[p];
-    }
-    // the pinned staging buffer is reused by the next call: wait for the copy
-    QSIM_CUDA(cudaStreamSynchronize(s->stream));
-    return SIM_OK;
+    if (M == 11) return run_staged<R, 11>(s, g);
+    if (M == 12) return run_staged<R, 12>(s, g);
+    if constexpr (sizeof(R) == 4) return run_staged<R, 13>(s, g);
+    return fail(SIM_EINVAL, "staged: complex128 tiles are at most 12 qubits");
 }
 
 }  // namespace
+
+double tile_cost(const std::vector<SGate> &g, int n, int dtype)
+{
+    double t = 0.0;
+    Program p;
+    if (dtype == SIM_C128) {
+        TilePlanner<double> plan(g, n, 12, 1, false, false);
+        while (plan.next(&p)) t += pass_cost<double>(p.tp);
+    } else {
+        TilePlanner<float> plan(g, n, 13, 2, false, false);
+        while (plan.next(&p)) t += pass_cost<float>(p.tp);
+    }
+    return t;
+}
+
+int run_tiles(qsim_state *s, const std::vector<SGate> &g)
+{
+    return s->dtype == SIM_C128 ? run_staged<double>(s, g, 12) : run_staged<float>(s, g, 13);
+}
 
 int describe_staged(int n, int dtype, const sim_gate *gates, size_t n_gates, int tile_qubits, int64_t *passes,
                     int64_t *ops, int64_t *layout_changes, int32_t *order, size_t order_cap, size_t *order_len)
@@ -265,6 +215,36 @@ int encode_staged(int n, int dtype, const sim_gate *gates, size_t n_gates, int t
     return SIM_OK;
 }
 
+int export_tile_programs(int n, int dtype, const sim_gate *gates, size_t n_gates, int tile_qubits, uint32_t *words,
+                         size_t words_cap, int32_t *info, size_t info_cap, size_t *n_words, size_t *n_passes)
+{
+    const bool c128 = dtype == SIM_C128;
+    int M = tile_qubits ? tile_qubits : (c128 ? 11 : 13);
+    if (M > n || M < 11 || M > (c128 ? 12 : 13)) return fail(SIM_EINVAL, "tile programs: no staged tile fits");
+    std::vector<SGate> g;
+    lower_renamed(gates, n_gates, n, &g);
+    const std::vector<Program> ps = compile_passes<double>(g, n, M, c128 ? 1 : 2);
+    size_t at = 0;
+    for (size_t p = 0; p < ps.size(); ++p) {
+        for (size_t k = 0; words && k < ps[p].words.size() && at + k < words_cap; ++k) words[at + k] = ps[p].words[k];
+        if (info && (p + 1) * SIM_TILE_PASS_INFO <= info_cap) {
+            int32_t *r = info + p * SIM_TILE_PASS_INFO;
+            for (int j = 0; j < SIM_TILE_PASS_INFO; ++j) r[j] = 0;
+            const uint64_t flip = ps[p].tp.flip;
+            const std::vector<int> &high = ps[p].pass.high;
+            const int32_t v[10] = {(int32_t)at, (int32_t)ps[p].words.size(), M, M - kTpThrBits, c128 ? 1 : 2,
+                                   ps[p].tp.start_layout, ps[p].tp.end_layout, (int32_t)(uint32_t)flip,
+                                   (int32_t)(uint32_t)(flip >> 32), (int32_t)high.size()};
+            for (int j = 0; j < 10; ++j) r[j] = v[j];
+            for (size_t i = 0; i < high.size() && i < 14; ++i) r[10 + i] = high[i];
+        }
+        at += ps[p].words.size();
+    }
+    if (n_words) *n_words = at;
+    if (n_passes) *n_passes = ps.size();
+    return SIM_OK;
+}
+
 int apply_circuit_staged(qsim_state *s, const sim_gate *gates, size_t n_gates, const sim_plan_opts &o)
 {
     const bool c128 = s->dtype == SIM_C128;
@@ -279,7 +259,7 @@ int apply_circuit_staged(qsim_state *s, const sim_gate *gates, size_t n_gates, c
         return SIM_OK;
     }
     std::vector<SGate> g;
-    lower_gates(gates, n_gates, &g);
+    lower_renamed(gates, n_gates, s->n, &g);
     if (g.empty()) return SIM_OK;
     return c128 ? run_staged<double>(s, g, M) : run_staged<float>(s, g, M);
 }

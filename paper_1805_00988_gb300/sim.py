@@ -269,6 +269,24 @@ def sim_plan_staged_ops(n: int, dtype: int, sim_gates: np.ndarray, tile_qubits: 
     return ops, info
 
 
+_sig("sim_plan_tile_programs", [_i32, _i32, P, _sz, _i32, P, _sz, P, _sz, P, P])
+
+
+def sim_plan_tile_programs(n: int, dtype: int, sim_gates: np.ndarray, tile_qubits: int = 0):
+    """The staged plan's tile programs (host only, FP64 tables): returns (words
+    as uint32, info as an int32 array of shape (passes, SIM_TILE_PASS_INFO))."""
+    g = np.ascontiguousarray(sim_gates, dtype=SIM_GATE_DTYPE)
+    nw, npass = ctypes.c_size_t(), ctypes.c_size_t()
+    check(_lib.sim_plan_tile_programs(n, dtype, g.ctypes.data_as(P), len(g), tile_qubits, None, 0, None, 0,
+                                      ctypes.byref(nw), ctypes.byref(npass)))
+    words = np.zeros(nw.value, dtype=np.uint32)
+    info = np.zeros((npass.value, SIM_TILE_PASS_INFO), dtype=np.int32)
+    check(_lib.sim_plan_tile_programs(n, dtype, g.ctypes.data_as(P), len(g), tile_qubits, words.ctypes.data_as(P),
+                                      len(words), info.ctypes.data_as(P), info.size, ctypes.byref(nw),
+                                      ctypes.byref(npass)))
+    return words, info
+
+
 def sim_plan_describe(n: int, dtype: int, sim_gates: np.ndarray, opts: sim_plan_opts):
     """Host-only: (passes, ops, layout_changes, order) of the staged schedule."""
     g = np.ascontiguousarray(sim_gates, dtype=SIM_GATE_DTYPE)
