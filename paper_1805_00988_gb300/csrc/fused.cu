@@ -30,6 +30,7 @@
 // records SIM_ETIMEOUT in a device status word, frees its tensor memory and
 // returns.
 #include <algorithm>
+#include <array>
 #include <cstring>
 #include <vector>
 
@@ -1719,6 +1720,120 @@ int describe_fused(int n, const sim_gate *gates, size_t n_gates, int k, int64_t 
 
 int fused_feature_depth() { return kFeatureDepth; }
 
+// ------------------------------------------------------------------ blocks and tiles
+// A block pass moves the state once for the gates of six qubits, whatever they
+// are; a register-tile pass once for those of thirteen, at a cost per gate.
+// So dense layers and CNOT ladders go faster in blocks and diagonal gates, Hadamards,
+// QFTs and permutations in tiles (26 qubits, 208-gate windows: Haar layers 2.5
+// against 3.0 ms, a U3 + CNOT ladder 2.5 against 5.4, graph-state edges 3.4
+// against 0.2-0.8, a QFT 8.4 against 3.3, phases 2.7 against 0.6).  The gate list
+// is cut into windows of about eight layers, both plans are costed for each
+// (on the host threads), and neighbouring windows with the same choice run as
+// one call.  complex128: 4-qubit blocks against tiles of 12 qubits.
+// Below these sizes the planning would not be paid back (0.5-0.9 ms).
+bool fused_mixes(int n, int dtype, int k)
+{
+    return dtype == SIM_C128 ? k == 4 && n >= 22 : k == 6 && n >= 26;
+}
+
+static int run_blocks(qsim_state *s, const std::vector<SGate> &g, int k)
+{
+    return k == 4 ? run_fused<4>(s, g, kRunDepth, false) : run_fused<6>(s, g, kRunDepth, false);
+}
+
+// 0 (blocks) or 1 (tiles) for each window of W gates of the first ng
+static std::vector<int> mixed_choice(const std::vector<SGate> &all, size_t ng, size_t W, int n, int dtype, int k)
+{
+    const size_t nw = (ng + W - 1) / W;
+    // one block pass on 2^26 amplitudes; times the blocks that run for each one
+    // the depth-1 search finds (it plans no further than it has to here: 0.5 ms
+    // a window); from 28 qubits on the planning of the run is hidden
+    const double block_us = dtype == SIM_C128 ? 0.84 * 520.0 : (n < 28 ? 0.8 : 0.72) * 190.0;
+    // a change of plan has to gain more than the estimates of a window are off
+    // (its own cost, the pool applied and no shared passes, is a fifth of that)
+    const double swap_us = dtype == SIM_C128 ? 4000.0 : 1500.0;
+    std::vector<double> tile(nw, 0.0), block(nw, 0.0);
+    auto window = [&](size_t w) {
+        return std::vector<SGate>(all.begin() + (long)(w * W), all.begin() + (long)std::min(ng, (w + 1) * W));
+    };
+    // A count of the gates is enough for most windows (microseconds per
+    // rotation, diagonal pair and masked exchange in tiles; rotations and pairs
+    // per block): both plans are costed only where masked exchanges decide,
+    // whose blocks depend on where they lie.
+    std::vector<char> exact(nw, 0);
+    const bool c128 = dtype == SIM_C128;
+    for (size_t w = 0; w < nw; ++w) {
+        double rot = 0, xch = 0, cz = 0, cp = 0;
+        const size_t end = std::min(ng, (w + 1) * W);
+        for (size_t i = w * W; i < end; ++i) {
+            const SGate &g = all[i];
+            if (g.xq() && !g.ctrl) rot += g.op == OP_XPERM ? 0 : 1;
+            else if (g.xq()) xch += 1;
+            else if (g.ctrl) (g.m[6] == -1.0 && g.m[7] == 0.0 ? cz : cp) += 1;
+        }
+        if (c128) {
+            tile[w] = 320 + 330 * rot + 80 * xch + 45 * cp + cz;
+            block[w] = std::max({block_us, block_us * rot / 6.0, block_us * (cz + cp) / 4.5});
+        } else {
+            tile[w] = 130 + 18.2 * rot + 38 * xch + 4 * cp + 0.5 * cz;
+            block[w] = std::max({block_us, (n < 28 ? 22.5 : 17.2) * rot, block_us * (cz + cp) / 9.0});
+        }
+        exact[w] = 10 * xch > (double)(end - w * W);
+    }
+    parallel_for(2 * nw, [&](size_t i) {
+        if (!exact[i / 2]) return;
+        const std::vector<SGate> g = window(i / 2);
+        if (i & 1) {
+            tile[i / 2] = tile_cost(g, n, dtype);
+        } else {
+            BlockPlanner planner(g, k, n, kFeatureDepth);
+            Block b;
+            int nb = 0;
+            while (planner.next(&b)) ++nb;
+            block[i / 2] = block_us * nb;
+        }
+    });
+    // the cheapest sequence of choices (0: blocks, 1: tiles)
+    std::vector<std::array<double, 2>> best(nw);
+    std::vector<std::array<int, 2>> from(nw);
+    for (size_t w = 0; w < nw; ++w)
+        for (int c = 0; c < 2; ++c) {
+            const double own = c ? tile[w] : block[w];
+            if (w == 0) {
+                best[w][c] = own;
+                from[w][c] = c;
+                continue;
+            }
+            const double stay = best[w - 1][c], turn = best[w - 1][1 - c] + swap_us;
+            best[w][c] = own + std::min(stay, turn);
+            from[w][c] = stay <= turn ? c : 1 - c;
+        }
+    std::vector<int> choice(nw, 0);
+    if (nw) choice[nw - 1] = best[nw - 1][1] < best[nw - 1][0] ? 1 : 0;
+    for (size_t w = nw; w-- > 1;) choice[w - 1] = from[w][choice[w]];
+    return choice;
+}
+
+static int run_mixed(qsim_state *s, const std::vector<SGate> &all, int k)
+{
+    // the renaming's last exchanges of places run as tile passes
+    size_t ng = all.size();
+    while (ng && all[ng - 1].op == OP_SWAP) --ng;
+    const size_t W = (size_t)std::max(64, 8 * s->n), nw = (ng + W - 1) / W;
+    const std::vector<int> choice = mixed_choice(all, ng, W, s->n, s->dtype, k);
+    for (size_t w = 0; w < nw;) {
+        size_t e = w + 1;
+        while (e < nw && choice[e] == choice[w]) ++e;
+        const size_t end = (e == nw && choice[w]) ? all.size() : std::min(ng, e * W);
+        const std::vector<SGate> g(all.begin() + (long)(w * W), all.begin() + (long)end);
+        if (int rc = choice[w] ? run_tiles(s, g) : run_blocks(s, g, k)) return rc;
+        w = e;
+    }
+    if (ng < all.size() && (nw == 0 || !choice[nw - 1]))
+        return run_tiles(s, std::vector<SGate>(all.begin() + (long)ng, all.end()));
+    return SIM_OK;
+}
+
 int apply_sgates_fused(qsim_state *s, const std::vector<SGate> &g, const double *sup, int k)
 {
     if (k < 3 || k > 6) return fail(SIM_EINVAL, "fused plan: fuse_k must be in 3..6");
@@ -1742,6 +1857,15 @@ int apply_circuit_fused(qsim_state *s, const sim_gate *gates, size_t n_gates, co
     if (c128 && k != 4) return fail(SIM_EUNSUPPORTED, "fused plan: complex128 states run 4-qubit blocks (fuse_k 4 or 0)");
     if (s->n < k + 7) return fail(SIM_EINVAL, "fused plan: needs n >= fuse_k + 7 (one CTA covers 128 rows)");
     std::vector<SGate> g;
+    if (fused_mixes(s->n, s->dtype, k)) {
+        lower_renamed(gates, n_gates, s->n, &g);
+        // unitary circuits only: what the blocks' scales refuse stays refused
+        bool unitary = true;
+        for (size_t i = 0; i < g.size() && unitary; ++i)
+            unitary = g[i].op == OP_SWAP || std::abs(sgate_norm_bound(g[i]) - 1.0) < 1e-6;
+        if (unitary) return run_mixed(s, g, k);
+        g.clear();
+    }
     lower_gates(gates, n_gates, &g);
     if (g.empty()) return SIM_OK;
     const bool multi = (o.flags & SIM_FLAG_MULTI_BLOCK_PASSES) != 0;

@@ -24,6 +24,8 @@ namespace qsim {
 
 namespace {
 
+constexpr int kConsultFrom = 26;   // complex64 registers below run 12-qubit tiles without asking the model
+
 struct Window {
     size_t first, count;
 };
@@ -101,12 +103,30 @@ int learned_choose(qsim_state *s, const sim_gate *gates, size_t n_gates, std::ve
     const size_t nw = win.size();
     // predicted log times of the feasible variants of some segments, the
     // feature rows in parallel on the host threads, one batched forward pass
+    // where the 6-qubit fused plan mixes in tile passes it holds the other
+    // variants' strengths: only the 13-qubit tile plan is weighed against it,
+    // and has to be predicted faster by more than the model's error
+    const bool mixes = fused_mixes(s->n, s->dtype, 6);
+    // there only windows where controlled exchanges (CNOT, Toffoli, ...) decide
+    // are in doubt: a count of the gates answers the others
+    std::vector<char> asked(nw, 1);
+    for (size_t w = 0; w < nw && mixes; ++w) {
+        size_t x = 0;
+        for (size_t k = win[w].first; k < win[w].first + win[w].count; ++k) {
+            const sim_gate &g = gates[k];
+            if (g.n_controls == 0) continue;
+            const PairGate p = make_pair_gate(g);
+            x += p.op == OP_DENSE || p.op == OP_ANTIDIAG || p.op == OP_XPERM || p.op == OP_SWAP;
+        }
+        asked[w] = 10 * x > win[w].count;
+    }
+    constexpr double kMixMargin = 0.845;
     struct Pred { size_t seg; int v; float p; };
     auto predict = [&](const std::vector<Window> &segs, std::vector<Pred> *out) -> int {
         std::vector<std::pair<size_t, int>> cand;
         for (size_t w = 0; w < segs.size(); ++w)
             for (int v = 0; v < SIM_VARIANTS; ++v)
-                if (feasible(s->n, s->dtype, v)) cand.push_back({w, v});
+                if (feasible(s->n, s->dtype, v) && asked[w] && (!mixes || v == 2 || v == 6)) cand.push_back({w, v});
         std::vector<float> feat(cand.size() * SIM_FEATURES);
         std::vector<char> ok(cand.size(), 0);
         parallel_for(cand.size(), [&](size_t r) {
@@ -125,13 +145,16 @@ int learned_choose(qsim_state *s, const sim_gate *gates, size_t n_gates, std::ve
         if (!out->empty())
             if (int rc = sim_mlp_forward((qsim_mlp *)s->cost_model, rows.data(), (int64_t)out->size(), pred.data(), 0))
                 return rc;
-        for (size_t r = 0; r < out->size(); ++r) (*out)[r].p = pred[r];
+        for (size_t r = 0; r < out->size(); ++r)
+            (*out)[r].p = pred[r] + (mixes && (*out)[r].v == 6 ? (float)std::log(kMixMargin) : 0.f);
         return SIM_OK;
     };
     std::vector<Pred> pw;
     if (int rc = predict(win, &pw)) return rc;
     std::vector<int> &best = *best_out;
     best.assign(nw, -1);
+    for (size_t w = 0; w < nw; ++w)
+        if (!asked[w]) best[w] = 6;
     std::vector<float> bestp(nw, 0.f);
     for (const Pred &x : pw)
         if (best[x.seg] < 0 || x.p < bestp[x.seg]) { best[x.seg] = x.v; bestp[x.seg] = x.p; }
@@ -149,7 +172,6 @@ int learned_choose(qsim_state *s, const sim_gate *gates, size_t n_gates, std::ve
     // whole circuit here: those feature rows cost more host time than the
     // windows' rows together.
     if (!agree && nw > 1) {
-        constexpr double kMixMargin = 0.845;
         std::vector<double> uni(SIM_VARIANTS, 0.0);
         std::vector<size_t> seen(SIM_VARIANTS, 0);
         for (const Pred &x : pw) {
@@ -214,6 +236,16 @@ int apply_circuit_learned(qsim_state *s, const sim_gate *gates, size_t n_gates, 
         for (size_t k = 0; k < n_gates; ++k)
             if (int rc = launch_pair_gate(s, make_pair_gate(gates[k]))) return rc;
         return SIM_OK;
+    }
+    if (s->n >= 12 && s->n < kConsultFrom) {
+        // 12-qubit tiles were the fastest variant of every window family here,
+        // or within 3 % of it, and asking the model costs 0.3-0.5 ms of a
+        // circuit that takes 0.4-7 ms (18-24 qubits)
+        s->last_plan.assign((n_gates + (size_t)std::max(64, 8 * s->n) - 1) / (size_t)std::max(64, 8 * s->n), 1);
+        sim_plan_opts so{};
+        so.plan = SIM_PLAN_STAGED;
+        so.tile_qubits = 12;
+        return apply_circuit_staged(s, gates, n_gates, so);
     }
     std::vector<int> best;
     if (int rc = learned_choose(s, gates, n_gates, &best)) return rc;
