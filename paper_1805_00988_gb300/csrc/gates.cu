@@ -195,6 +195,41 @@ __device__ __forceinline__ void stv(R *st, uint64_t amp, const typename Vec<R, V
 
 constexpr int kThreads = 256;
 
+// Small registers are bound by the gap between launches and by how few SMs a
+// gate reaches, not by bytes (5.2 us a gate at 14 qubits):
+//  - a gate's kernel may be launched while the one before it still runs
+//    (programmatic stream serialisation) and waits for it before it touches
+//    the state, so launch latency overlaps the previous gate;
+//  - U = 1 with 64-thread blocks when the usual blocks would leave SMs idle
+//    (fewer than one a SM): a complex128 dense gate of 14 qubits ran its FP64
+//    work on 16 SMs.
+// 14 qubits: 5.2 -> 1.9 us a gate complex128, 4.1 -> 1.9 complex64; 24 qubits
+// still gain the latency (31.2 -> 28.8 us).
+constexpr int kSmallThreads = 64;
+constexpr uint64_t kSpread = 152;
+
+__device__ __forceinline__ void pdl_enter()
+{
+    cudaTriggerProgrammaticLaunchCompletion();
+    cudaGridDependencySynchronize();
+}
+
+// launch fn with the programmatic attribute on the handle's stream
+template <typename... P, typename... A>
+void launch_pdl(cudaStream_t stream, void (*fn)(P...), uint64_t blocks, int threads, A... args)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, fn, P(args)...);       // errors: launch_end
+}
+
 // Two separate vector accesses per item: the lo amplitudes at base | lo_off
 // and the hi amplitudes at base | hi_off.  VEC neighbouring amplitudes per
 // vector (all involved bits are >= log2(VEC)).
@@ -202,12 +237,14 @@ template <typename R, int VEC, int OP, int U>
 __global__ void __launch_bounds__(kThreads) k_pair_split(R *__restrict__ st, PairArgs a, Coef<R> c)
 {
     using V = typename Vec<R, VEC>::T;
-    const uint64_t first = (uint64_t)blockIdx.x * (uint64_t)(kThreads * U) + threadIdx.x;
+    constexpr int T = U == 1 ? kSmallThreads : kThreads;
+    const uint64_t first = (uint64_t)blockIdx.x * (uint64_t)(T * U) + threadIdx.x;
+    pdl_enter();
     V lo[U], hi[U];
     uint64_t base[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-        const uint64_t w = first + (uint64_t)u * kThreads;
+        const uint64_t w = first + (uint64_t)u * T;
         base[u] = ~0ull;
         if (w < a.n_items) {
             base[u] = insert_zeros(w * VEC, a) | a.set_mask;
@@ -237,12 +274,14 @@ __global__ void __launch_bounds__(kThreads) k_pair_split(R *__restrict__ st, Pai
 template <int OP, int U>
 __global__ void __launch_bounds__(kThreads) k_pair_inner(float *__restrict__ st, PairArgs a, Coef<float> c)
 {
-    const uint64_t first = (uint64_t)blockIdx.x * (uint64_t)(kThreads * U) + threadIdx.x;
+    constexpr int T = U == 1 ? kSmallThreads : kThreads;
+    const uint64_t first = (uint64_t)blockIdx.x * (uint64_t)(T * U) + threadIdx.x;
+    pdl_enter();
     float4 v[U];
     uint64_t base[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-        const uint64_t w = first + (uint64_t)u * kThreads;
+        const uint64_t w = first + (uint64_t)u * T;
         base[u] = ~0ull;
         if (w < a.n_items) {
             base[u] = insert_zeros(w, a) | a.set_mask;
@@ -268,22 +307,26 @@ Coef<R> make_coef(const double m[8])
 }
 
 template <typename R, int VEC, int OP, int U>
-cudaError_t go_split(qsim_state *s, const PairArgs &a, const Coef<R> &c)
+void go_split(qsim_state *s, const PairArgs &a, const Coef<R> &c)
 {
-    const uint64_t per = (uint64_t)kThreads * U;
-    const uint64_t blocks = (a.n_items + per - 1) / per;
-    k_pair_split<R, VEC, OP, U><<<(unsigned)blocks, kThreads, 0, s->stream>>>((R *)s->amps, a, c);
-    return cudaSuccess;
+    const uint64_t per = (uint64_t)kThreads * U, blocks = (a.n_items + per - 1) / per;
+    if (blocks >= kSpread)
+        launch_pdl(s->stream, k_pair_split<R, VEC, OP, U>, blocks, kThreads, (R *)s->amps, a, c);
+    else
+        launch_pdl(s->stream, k_pair_split<R, VEC, OP, 1>, (a.n_items + kSmallThreads - 1) / kSmallThreads,
+                   kSmallThreads, (R *)s->amps, a, c);
 }
 
 template <int OP>
-cudaError_t go_inner(qsim_state *s, const PairArgs &a, const Coef<float> &c)
+void go_inner(qsim_state *s, const PairArgs &a, const Coef<float> &c)
 {
     constexpr int U = 4;
-    const uint64_t per = (uint64_t)kThreads * U;
-    const uint64_t blocks = (a.n_items + per - 1) / per;
-    k_pair_inner<OP, U><<<(unsigned)blocks, kThreads, 0, s->stream>>>((float *)s->amps, a, c);
-    return cudaSuccess;
+    const uint64_t per = (uint64_t)kThreads * U, blocks = (a.n_items + per - 1) / per;
+    if (blocks >= kSpread)
+        launch_pdl(s->stream, k_pair_inner<OP, U>, blocks, kThreads, (float *)s->amps, a, c);
+    else
+        launch_pdl(s->stream, k_pair_inner<OP, 1>, (a.n_items + kSmallThreads - 1) / kSmallThreads, kSmallThreads,
+                   (float *)s->amps, a, c);
 }
 
 template <typename R, int VEC, int U>
