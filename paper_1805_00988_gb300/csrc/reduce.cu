@@ -487,29 +487,74 @@ __global__ void __launch_bounds__(kRedThreads) k_final_sum(const double *__restr
 }
 
 // ---------------------------------------------------------------- probabilities
+// 16-byte vectors of the state (two complex64 amplitudes, one complex128), four
+// in flight a thread; HBM-bound (28 qubits complex64: 3.2 GB).  aligned: the
+// output takes whole-vector stores.
 template <typename R, typename O>
-__global__ void k_probabilities(const R *__restrict__ st, uint64_t N, O *__restrict__ p)
+__global__ void __launch_bounds__(256) k_probabilities(const R *__restrict__ st, uint64_t nvec, O *__restrict__ p,
+                                                       bool aligned)
 {
-    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N;
-         i += (uint64_t)gridDim.x * blockDim.x) {
-        const R re = st[2 * i], im = st[2 * i + 1];
-        if (sizeof(O) == sizeof(R)) p[i] = (O)(re * re + im * im);
-        else p[i] = (O)sq<R>(re, im);
+    constexpr int A = sizeof(R) == 4 ? 2 : 1;          // amplitudes per vector
+    constexpr int U = 4;
+    struct alignas(16) Vec { R x[2 * A]; };
+    struct alignas(A * sizeof(O)) Out { O x[A]; };
+    const uint64_t step = (uint64_t)gridDim.x * blockDim.x;
+    for (uint64_t i0 = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i0 < nvec; i0 += U * step) {
+        Vec v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (i0 + u * step < nvec) v[u] = reinterpret_cast<const Vec *>(st)[i0 + u * step];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const uint64_t i = i0 + u * step;
+            if (i >= nvec) break;
+            Out o;
+#pragma unroll
+            for (int a = 0; a < A; ++a) {
+                const R re = v[u].x[2 * a], im = v[u].x[2 * a + 1];
+                if (sizeof(O) == sizeof(R)) o.x[a] = (O)(re * re + im * im);
+                else o.x[a] = (O)sq<R>(re, im);
+            }
+            if (aligned) {
+                reinterpret_cast<Out *>(p)[i] = o;
+            } else {
+#pragma unroll
+                for (int a = 0; a < A; ++a) p[A * i + a] = o.x[a];
+            }
+        }
     }
 }
 
 // ---------------------------------------------------------------- collapse
+// 16-byte vectors, four in flight a thread: the kept half is read, scaled and
+// written, the other half only written (HBM-bound).
 template <typename R>
-__global__ void k_collapse(R *__restrict__ st, uint64_t N, int q, int outcome, R scale)
+__global__ void __launch_bounds__(256) k_collapse(R *__restrict__ st, uint64_t nvec, int q, int outcome, R scale)
 {
-    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N;
-         i += (uint64_t)gridDim.x * blockDim.x) {
-        if ((int)((i >> q) & 1ull) == outcome) {
-            st[2 * i] *= scale;
-            st[2 * i + 1] *= scale;
-        } else {
-            st[2 * i] = (R)0;
-            st[2 * i + 1] = (R)0;
+    constexpr int A = sizeof(R) == 4 ? 2 : 1;
+    constexpr int U = 4;
+    struct alignas(16) Vec { R x[2 * A]; };
+    Vec *s = reinterpret_cast<Vec *>(st);
+    const uint64_t step = (uint64_t)gridDim.x * blockDim.x;
+    const int qv = q - (A - 1);                        // the qubit's bit of a vector index, -1: inside the vector
+    for (uint64_t i0 = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i0 < nvec; i0 += U * step) {
+        Vec v[U];
+        bool keep[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const uint64_t i = i0 + u * step;
+            keep[u] = qv < 0 || (int)((i >> qv) & 1ull) == outcome;
+            if (keep[u] && i < nvec) v[u] = s[i];
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const uint64_t i = i0 + u * step;
+            if (i >= nvec) break;
+            Vec o;
+#pragma unroll
+            for (int e = 0; e < 2 * A; ++e)
+                o.x[e] = (keep[u] && (qv >= 0 || (e >> 1) == outcome)) ? v[u].x[e] * scale : (R)0;
+            s[i] = o;
         }
     }
 }
@@ -1098,14 +1143,16 @@ int reduce_norm_device(qsim_state *s)
 int launch_probabilities(qsim_state *s, void *dev_out, int out_real)
 {
     const uint64_t N = 1ull << s->n;
-    const unsigned g = grid_for(N, 256, s->num_sms);
+    const uint64_t nvec = (s->dtype == SIM_C128) ? N : N / 2;
+    const unsigned g = grid_for(nvec, 256, s->num_sms);
+    const bool aligned = ((uintptr_t)dev_out & 15u) == 0;
     launch_begin(s, KC_PROB, (double)s->bytes + (double)N * (out_real == SIM_F64 ? 8.0 : 4.0));
     if (s->dtype == SIM_C128) {
-        if (out_real == SIM_F64) k_probabilities<double, double><<<g, 256, 0, s->stream>>>((const double *)s->amps, N, (double *)dev_out);
-        else k_probabilities<double, float><<<g, 256, 0, s->stream>>>((const double *)s->amps, N, (float *)dev_out);
+        if (out_real == SIM_F64) k_probabilities<double, double><<<g, 256, 0, s->stream>>>((const double *)s->amps, nvec, (double *)dev_out, aligned);
+        else k_probabilities<double, float><<<g, 256, 0, s->stream>>>((const double *)s->amps, nvec, (float *)dev_out, aligned);
     } else {
-        if (out_real == SIM_F64) k_probabilities<float, double><<<g, 256, 0, s->stream>>>((const float *)s->amps, N, (double *)dev_out);
-        else k_probabilities<float, float><<<g, 256, 0, s->stream>>>((const float *)s->amps, N, (float *)dev_out);
+        if (out_real == SIM_F64) k_probabilities<float, double><<<g, 256, 0, s->stream>>>((const float *)s->amps, nvec, (double *)dev_out, aligned);
+        else k_probabilities<float, float><<<g, 256, 0, s->stream>>>((const float *)s->amps, nvec, (float *)dev_out, aligned);
     }
     return launch_end(s, "probabilities");
 }
@@ -1113,12 +1160,13 @@ int launch_probabilities(qsim_state *s, void *dev_out, int out_real)
 int launch_collapse(qsim_state *s, int qubit, int outcome, double scale)
 {
     const uint64_t N = 1ull << s->n;
-    const unsigned g = grid_for(N, 256, s->num_sms);
+    const uint64_t nvec = (s->dtype == SIM_C128) ? N : N / 2;
+    const unsigned g = grid_for(nvec, 256, s->num_sms);
     launch_begin(s, KC_COLLAPSE, 1.5 * (double)s->bytes);
     if (s->dtype == SIM_C128)
-        k_collapse<double><<<g, 256, 0, s->stream>>>((double *)s->amps, N, qubit, outcome, scale);
+        k_collapse<double><<<g, 256, 0, s->stream>>>((double *)s->amps, nvec, qubit, outcome, scale);
     else
-        k_collapse<float><<<g, 256, 0, s->stream>>>((float *)s->amps, N, qubit, outcome, (float)scale);
+        k_collapse<float><<<g, 256, 0, s->stream>>>((float *)s->amps, nvec, qubit, outcome, (float)scale);
     return launch_end(s, "collapse");
 }
 
