@@ -129,7 +129,11 @@ __global__ void __launch_bounds__(kTpThr, (tile_ctas<float, M>()))
         }
 
         const uint4 *prog = progs + ps.prog0;
-        const int nunits = ps.nunits;
+        // the first pass finds |0...0>: every tile but the first is zero and
+        // stays so under gates that act inside tiles, so it runs no program
+        // (a fifth to a third of a large circuit's tiles)
+        const bool zero = it.pass == 0 && it.tile != 0;
+        const int nunits = zero ? 0 : ps.nunits;
         prog_stage(prog, nunits, tid, sp);
         uint64_t base = tile_base(ps.geo, (uint32_t)it.tile);
         float *st = reinterpret_cast<float *>(scratch + c.state0);
@@ -144,7 +148,7 @@ __global__ void __launch_bounds__(kTpThr, (tile_ctas<float, M>()))
             tile_load<M, RB, 2, true>(ps.start_layout, v, st, ps.geo, tid, base);
         }
         __syncthreads();
-        run_program<float, M, kFull>(v, prog, nunits, (uint32_t)it.tile, tid, sm, sp);
+        if (!zero) run_program<float, M, kFull>(v, prog, nunits, (uint32_t)it.tile, tid, sm, sp);
 
         if (it.pass + 1 < c.npass) {
             // addresses formed again instead of being held live across the program
