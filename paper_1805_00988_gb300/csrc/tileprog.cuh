@@ -1157,7 +1157,14 @@ inline bool split_general(const double m[8], cplx *p, cplx *q, cplx *a, cplx *b,
 template <typename R>
 class TileCompiler {
 public:
-    TileCompiler(int n, int M, int VEC) : pool(n), n_(n), M_(M), RB_(M - kTpThrBits), RA_(1 << (M - kTpThrBits)), VEC_(VEC) {}
+    TileCompiler(int n, int M, int VEC) : pool(n), n_(n), M_(M), RB_(M - kTpThrBits), RA_(1 << (M - kTpThrBits)), VEC_(VEC)
+    {
+        for (int l = 0; l < 4; ++l) {
+            io_[l] = io_layout(M_, RB_, VEC_, l);
+            for (int j = 0; j < RB_; ++j) lreg_[l][j] = l < n_layouts(M_, RB_) ? reg_local(M_, RB_, VEC_, l, j) : 0;
+            for (int i = 0; i < kTpThrBits; ++i) lthr_[l][i] = l < n_layouts(M_, RB_) ? thr_local(M_, RB_, VEC_, l, i) : 0;
+        }
+    }
 
     DiagPool pool;
 
@@ -1183,7 +1190,7 @@ public:
     void set_layout(int l)
     {
         if (l == layout_) return;
-        if (!started_ && !queued_ && pre_.empty() && !tab_used_ && io_layout(M_, RB_, VEC_, l)) {
+        if (!started_ && !queued_ && pre_.empty() && !tab_used_ && io_[l]) {
             // nothing ran yet: load in this layout
             layout_ = l;
             out_.start_layout = l;
@@ -1238,7 +1245,7 @@ public:
         flush_signs();
         if (!(last && unit_ok)) {                  // <sum Z> does not depend on where the qubits are
             if (loc_ != home_) restore_places();
-            if (!io_layout(M_, RB_, VEC_, layout_)) set_layout(0);
+            if (!io_[layout_]) set_layout(0);
         }
         out_.end_layout = layout_;
         out_.flip = flip_;
@@ -1249,6 +1256,8 @@ public:
 
 private:
     int n_, M_, RB_, RA_, VEC_;
+    bool io_[4];                          // layouts the pass may load and store in
+    int lreg_[4][8], lthr_[4][kTpThrBits];   // their local bits
     std::vector<int> loc_, outbit_;       // per qubit: local bit (-1: outside the tile), bit of the tile index
     std::vector<int> home_;               // loc_ as the state is stored
     std::vector<int> reg_, thr_;          // per qubit: register / thread bit of the current layout, -1 if none
@@ -1269,16 +1278,17 @@ private:
         reg_.assign((size_t)n_, -1);
         thr_.assign((size_t)n_, -1);
         regq_.assign((size_t)RB_, -1);
-        std::vector<int> qof((size_t)M_, -1);
+        int qof[16];
+        for (int b = 0; b < 16; ++b) qof[b] = -1;
         for (int q = 0; q < n_; ++q)
-            if (loc_[q] >= 0) qof[(size_t)loc_[q]] = q;
+            if (loc_[q] >= 0) qof[loc_[q]] = q;
         for (int j = 0; j < RB_; ++j) {
-            const int q = qof[(size_t)reg_local(M_, RB_, VEC_, layout_, j)];
+            const int q = qof[lreg_[layout_][j]];
             regq_[(size_t)j] = q;
             if (q >= 0) reg_[(size_t)q] = j;
         }
         for (int i = 0; i < kTpThrBits; ++i) {
-            const int q = qof[(size_t)thr_local(M_, RB_, VEC_, layout_, i)];
+            const int q = qof[lthr_[layout_][i]];
             if (q >= 0) thr_[(size_t)q] = i;
         }
     }
@@ -1293,7 +1303,7 @@ private:
     }
     void reset_group()
     {
-        tab_.assign((size_t)RA_, 1.0);
+        if (tab_used_ || tab_.size() != (size_t)RA_) tab_.assign((size_t)RA_, 1.0);
         tab_used_ = false;
         pre_.clear();
         queued_ = 0;
@@ -1360,7 +1370,7 @@ private:
                 for (cplx &c : tab_) c = times(c, s);
             pool.g = (s == pool.g) ? cplx(1.0) : pool.g / s;
             o.arg = real ? GD_REAL : GD_CPLX;
-            o.tab = tab_;
+            o.tab.swap(tab_);              // a fresh one at the next reset
         }
         pre_.push_back(std::move(o));
     }
@@ -1403,6 +1413,7 @@ private:
             TpOp o;
             o.op = IR_SHEARS;
             o.arg = queued_;
+            o.tab.reserve((size_t)RB_);
             for (int j = 0; j < RB_; ++j)
                 o.tab.push_back(((queued_ >> j) & 1u) ? cplx(sa_[j], sb_[j]) : cplx(0.0));
             emit(std::move(o));
@@ -1458,7 +1469,7 @@ private:
     {
         int to = 0;
         for (int l = 1; l < n_layouts(M_, RB_); ++l)
-            if (io_layout(M_, RB_, VEC_, l)) to = l;
+            if (io_[l]) to = l;
         auto weight = [&](int local) {
             int src = local;
             for (int q = 0; q < n_; ++q)
@@ -1468,8 +1479,8 @@ private:
         TpOp o;
         o.op = IR_PERM;
         o.arg = (uint32_t)(layout_ | (to << 2));
-        for (int i = 0; i < kTpThrBits; ++i) o.words.push_back(weight(thr_local(M_, RB_, VEC_, to, i)));
-        for (int j = 0; j < RB_; ++j) o.words.push_back(weight(reg_local(M_, RB_, VEC_, to, j)));
+        for (int i = 0; i < kTpThrBits; ++i) o.words.push_back(weight(lthr_[to][i]));
+        for (int j = 0; j < RB_; ++j) o.words.push_back(weight(lreg_[to][j]));
         emit(std::move(o));
         loc_ = home_;
         layout_ = to;
@@ -1907,6 +1918,7 @@ private:
         pool.g = 1.0;
         if (!singles.empty()) {
             pre_.push_back(make_ramp(-1, singles, 1.0, tab_used_ ? &tab_ : nullptr, true));
+            tab_.assign((size_t)RA_, 1.0);
             tab_used_ = false;
         }
         close_group();
@@ -1969,14 +1981,15 @@ public:
             stage = std::max(stage, o.op);
         }
         close();
-        std::vector<uint32_t> w(4, 0u);
-        put(w, TP_END);
+        w_.assign(4, 0u);
+        put(w_, TP_END);
     }
 
 private:
     std::vector<uint32_t> *out_;
     size_t first_;
     bool dirty_ = false;           // signs may be pending
+    std::vector<uint32_t> w_;      // the operation being packed
 
     static void real(std::vector<uint32_t> *w, double v)
     {
@@ -2028,7 +2041,8 @@ private:
     }
     void group(const std::vector<const TpOp *> &ops)
     {
-        std::vector<uint32_t> w(4, 0u);
+        std::vector<uint32_t> &w = w_;
+        w.assign(4, 0u);
         uint32_t head = TP_GROUP, nz = 0;
         for (const TpOp *o : ops)
             if (o->op == IR_Z) {
@@ -2064,7 +2078,8 @@ private:
     }
     void single(const TpOp &o)
     {
-        std::vector<uint32_t> w(4, 0u);
+        std::vector<uint32_t> &w = w_;
+        w.assign(4, 0u);
         w[1] = o.thr;
         w[2] = o.out;
         w[3] = o.place;
@@ -2103,8 +2118,13 @@ void schedule_pass(TileCompiler<R> &tc, const Pass &ps, const std::vector<SGate>
     const size_t P = ps.members.size();
     enum { DIAG, LABEL, ROT, MASKED };
     std::vector<uint8_t> kind(P), lmask(P, 0);
-    std::vector<int> indeg(P, 0), lastx(64, -1);
-    std::vector<std::vector<int>> succ(P), since(64);
+    std::vector<int> indeg(P, 0);
+    int lastx[64], since[64];              // per qubit: last exchange, list of the diagonal gates after it
+    for (int q = 0; q < 64; ++q) lastx[q] = since[q] = -1;
+    struct Link { int item, next; };
+    std::vector<Link> links;               // the lists: successors of a gate, diagonal gates of a qubit
+    links.reserve(8 * P);
+    std::vector<int> succ(P, -1);
     uint8_t lq[64];
     for (int q = 0; q < 64; ++q) lq[q] = 0;
     auto layouts_of = [&](int local) {
@@ -2116,7 +2136,8 @@ void schedule_pass(TileCompiler<R> &tc, const Pass &ps, const std::vector<SGate>
     for (int q = 0; q < kLow; ++q) lq[q] = layouts_of(q);
     for (size_t i = 0; i < ps.high.size(); ++i) lq[ps.high[i]] = layouts_of(kLow + (int)i);
     auto edge = [&](int a, int b) {
-        succ[(size_t)a].push_back(b);
+        links.push_back(Link{b, succ[(size_t)a]});
+        succ[(size_t)a] = (int)links.size() - 1;
         ++indeg[(size_t)b];
     };
     for (size_t i = 0; i < P; ++i) {
@@ -2128,23 +2149,27 @@ void schedule_pass(TileCompiler<R> &tc, const Pass &ps, const std::vector<SGate>
         if (x) lmask[i] = lq[s.target];
         for (uint64_t m = d; m; m &= m - 1) {
             const int q = __builtin_ctzll(m);
-            if (lastx[(size_t)q] >= 0) edge(lastx[(size_t)q], (int)i);
-            since[(size_t)q].push_back((int)i);
+            if (lastx[q] >= 0) edge(lastx[q], (int)i);
+            links.push_back(Link{(int)i, since[q]});
+            since[q] = (int)links.size() - 1;
         }
         for (uint64_t m = x; m; m &= m - 1) {
             const int q = __builtin_ctzll(m);
-            if (lastx[(size_t)q] >= 0 && since[(size_t)q].empty()) edge(lastx[(size_t)q], (int)i);
-            for (int j : since[(size_t)q]) edge(j, (int)i);
-            since[(size_t)q].clear();
-            lastx[(size_t)q] = (int)i;
+            if (lastx[q] >= 0 && since[q] < 0) edge(lastx[q], (int)i);
+            for (int l = since[q]; l >= 0; l = links[(size_t)l].next) {
+                const int before = links[(size_t)l].item;   // (edge grows links)
+                edge(before, (int)i);
+            }
+            since[q] = -1;
+            lastx[q] = (int)i;
         }
     }
     std::vector<int> ready, now;
     for (size_t i = 0; i < P; ++i)
         if (!indeg[i]) ready.push_back((int)i);
     auto done = [&](int i) {
-        for (int j : succ[(size_t)i])
-            if (--indeg[(size_t)j] == 0) ready.push_back(j);
+        for (int l = succ[(size_t)i]; l >= 0; l = links[(size_t)l].next)
+            if (--indeg[(size_t)links[(size_t)l].item] == 0) ready.push_back(links[(size_t)l].item);
     };
     auto run = [&](int i, int l) {
         tc.gate(g[(size_t)ps.members[(size_t)i]], l);
