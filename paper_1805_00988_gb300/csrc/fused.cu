@@ -30,7 +30,6 @@
 // records SIM_ETIMEOUT in a device status word, frees its tensor memory and
 // returns.
 #include <algorithm>
-#include <array>
 #include <cstring>
 #include <vector>
 
@@ -1731,9 +1730,13 @@ int fused_feature_depth() { return kFeatureDepth; }
 // (on the host threads), and neighbouring windows with the same choice run as
 // one call.  complex128: 4-qubit blocks against tiles of 12 qubits.
 // Below these sizes the planning would not be paid back (0.5-0.9 ms).
-bool fused_mixes(int n, int dtype, int k)
+// complex128 under the learned plan mixes at every size: up to 19 qubits a
+// block pass costs more to prepare on the host than to run, and tiles alone take less for
+// every family (12 Haar layers, 14 / 19 qubits: 482 / 1092 us against 940 / 1629; QFT
+// 150 / 260 against 442 / 1195; U3 + CNOT ladder 571 / 1178 against 714 / 1557).
+bool fused_mixes(int n, int dtype, int k, bool learned)
 {
-    return dtype == SIM_C128 ? k == 4 && n >= 22 : k == 6 && n >= 26;
+    return dtype == SIM_C128 ? k == 4 && (learned || n >= 22) : k == 6 && n >= 26;
 }
 
 static int run_blocks(qsim_state *s, const std::vector<SGate> &g, int k)
@@ -1773,12 +1776,13 @@ static std::vector<int> mixed_choice(const std::vector<SGate> &all, size_t ng, s
         }
         if (c128) {
             tile[w] = 320 + 330 * rot + 80 * xch + 45 * cp + cz;
-            block[w] = std::max({block_us, block_us * rot / 6.0, block_us * (cz + cp) / 4.5});
+            block[w] = std::max({block_us, block_us * (rot + (n < 22 ? xch : 0)) / 6.0, block_us * (cz + cp) / 4.5});
         } else {
             tile[w] = 130 + 18.2 * rot + 38 * xch + 4 * cp + 0.5 * cz;
             block[w] = std::max({block_us, (n < 28 ? 22.5 : 17.2) * rot, block_us * (cz + cp) / 9.0});
         }
-        exact[w] = 10 * xch > (double)(end - w * W);
+        // (complex128 below 22 qubits: 0.2 ms of costing on a circuit of 2 ms)
+        exact[w] = 10 * xch > (double)(end - w * W) && !(c128 && n < 22);
     }
     parallel_for(2 * nw, [&](size_t i) {
         if (!exact[i / 2]) return;
@@ -1816,6 +1820,7 @@ static std::vector<int> mixed_choice(const std::vector<SGate> &all, size_t ng, s
 
 static int run_mixed(qsim_state *s, const std::vector<SGate> &all, int k)
 {
+    if (s->dtype == SIM_C128 && s->n < 20) return run_tiles(s, all);
     // the renaming's last exchanges of places run as tile passes
     size_t ng = all.size();
     while (ng && all[ng - 1].op == OP_SWAP) --ng;
@@ -1857,7 +1862,8 @@ int apply_circuit_fused(qsim_state *s, const sim_gate *gates, size_t n_gates, co
     if (c128 && k != 4) return fail(SIM_EUNSUPPORTED, "fused plan: complex128 states run 4-qubit blocks (fuse_k 4 or 0)");
     if (s->n < k + 7) return fail(SIM_EINVAL, "fused plan: needs n >= fuse_k + 7 (one CTA covers 128 rows)");
     std::vector<SGate> g;
-    if (fused_mixes(s->n, s->dtype, k)) {
+    const bool multi = (o.flags & SIM_FLAG_MULTI_BLOCK_PASSES) != 0;
+    if (!multi && fused_mixes(s->n, s->dtype, k, o.plan == SIM_PLAN_LEARNED)) {
         lower_renamed(gates, n_gates, s->n, &g);
         // unitary circuits only: what the blocks' scales refuse stays refused
         bool unitary = true;
@@ -1868,7 +1874,6 @@ int apply_circuit_fused(qsim_state *s, const sim_gate *gates, size_t n_gates, co
     }
     lower_gates(gates, n_gates, &g);
     if (g.empty()) return SIM_OK;
-    const bool multi = (o.flags & SIM_FLAG_MULTI_BLOCK_PASSES) != 0;
     switch (k) {
     case 3: return run_fused<3>(s, g, kRunDepth, multi);
     case 4: return run_fused<4>(s, g, kRunDepth, multi);

@@ -8,6 +8,7 @@
 #include <atomic>
 #include <thread>
 #include <algorithm>
+#include <array>
 #include <memory>
 #include <vector>
 
@@ -213,7 +214,8 @@ int run_tiles(qsim_state *s, const std::vector<SGate> &g);
 double tile_cost(const std::vector<SGate> &g, int n, int dtype);
 // registers from this size on: the fused plan with the largest blocks takes
 // tile passes for the stretches they are predicted to be faster on
-bool fused_mixes(int n, int dtype, int k);
+bool fused_mixes(int n, int dtype, int k, bool learned);
+bool learned_tiles_only(int n, int dtype);
 int apply_circuit_learned(qsim_state *s, const sim_gate *gates, size_t n_gates, const sim_plan_opts &o);
 int plan_features(int n, int dtype, const sim_gate *gates, size_t n_gates, int v, float *out);
 // the learned plan's variant per window for a complex64 register with a cost

@@ -106,7 +106,7 @@ int learned_choose(qsim_state *s, const sim_gate *gates, size_t n_gates, std::ve
     // where the 6-qubit fused plan mixes in tile passes it holds the other
     // variants' strengths: only the 13-qubit tile plan is weighed against it,
     // and has to be predicted faster by more than the model's error
-    const bool mixes = fused_mixes(s->n, s->dtype, 6);
+    const bool mixes = fused_mixes(s->n, s->dtype, 6, true);
     // there only windows where controlled exchanges (CNOT, Toffoli, ...) decide
     // are in doubt: a count of the gates answers the others
     std::vector<char> asked(nw, 1);
@@ -193,6 +193,12 @@ int learned_choose(qsim_state *s, const sim_gate *gates, size_t n_gates, std::ve
     return SIM_OK;
 }
 
+// registers on which the learned plan runs tiles whatever the circuit
+bool learned_tiles_only(int n, int dtype)
+{
+    return dtype == SIM_C128 ? n >= 11 && n < 20 : n >= 12 && n < kConsultFrom;
+}
+
 int apply_circuit_learned(qsim_state *s, const sim_gate *gates, size_t n_gates, const sim_plan_opts &o)
 {
     if (!s->cost_model) {
@@ -222,13 +228,14 @@ int apply_circuit_learned(qsim_state *s, const sim_gate *gates, size_t n_gates, 
         // tensor cores as exact integer digit-plane products (fused64.cu).
         // Measured at 30 qubits (Haar layers + CZ, depth 20): fused 1276 ms
         // against 12837 ms per gate; 28-qubit QFT: 253 against 351 ms.  So the
-        // fused plan runs wherever a 4-qubit block's tile fits (n >= 11), the
+        // fused plan, with register tiles where those are faster (its mixed
+        // form), runs wherever a 4-qubit block's tile fits (n >= 11), the
         // per-gate plan below that; the model (trained on complex64 timings)
         // is not consulted.
         if (s->n >= 11) {
             s->last_plan.assign(1, 4);
             sim_plan_opts fo{};
-            fo.plan = SIM_PLAN_FUSED;
+            fo.plan = SIM_PLAN_LEARNED;
             fo.fuse_k = 4;
             return apply_circuit_fused(s, gates, n_gates, fo);
         }
@@ -237,14 +244,15 @@ int apply_circuit_learned(qsim_state *s, const sim_gate *gates, size_t n_gates, 
             if (int rc = launch_pair_gate(s, make_pair_gate(gates[k]))) return rc;
         return SIM_OK;
     }
-    if (s->n >= 12 && s->n < kConsultFrom) {
+    if (learned_tiles_only(s->n, s->dtype)) {
         // 12-qubit tiles were the fastest variant of every window family here,
         // or within 3 % of it, and asking the model costs 0.3-0.5 ms of a
-        // circuit that takes 0.4-7 ms (18-24 qubits)
+        // circuit that takes 0.4-7 ms (18-24 qubits).  Up to 18 qubits the
+        // tiles are of 11 (the staged plan's rule; reported as variant 1, too)
         s->last_plan.assign((n_gates + (size_t)std::max(64, 8 * s->n) - 1) / (size_t)std::max(64, 8 * s->n), 1);
         sim_plan_opts so{};
         so.plan = SIM_PLAN_STAGED;
-        so.tile_qubits = 12;
+        so.tile_qubits = s->n <= 18 ? 11 : 12;
         return apply_circuit_staged(s, gates, n_gates, so);
     }
     std::vector<int> best;
