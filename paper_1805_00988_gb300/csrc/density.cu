@@ -14,7 +14,11 @@
 //   - a single-qubit channel rho -> sum_m K_m rho K_m^dagger on qubit t is a
 //     4 x 4 matrix on register qubits (t + n, t):
 //       S[2r + c][2r' + c'] = sum_m K_m[r][r'] conj(K_m[c][c']),
-//     applied by k_superop, one pass over the register;
+//     applied by k_superop, one pass over the register.  The named channels'
+//     matrices are real and connect only r = c entries with each other and
+//     r != c entries with each other (k_channels); under the staged and the learned plan
+//     the channels between two gates of a qubit are multiplied into one matrix, and
+//     one pass applies those of two qubits;
 //   - p_j = Re rho[j][j] sits at register index j (2^n + 1): trace, <sum Z>,
 //     measurement and sampling read the diagonal into a complex128 vector of
 //     2^n amplitudes sqrt(max(p_j, 0)) and run the state-vector reductions
@@ -33,6 +37,7 @@ namespace qsim {
 namespace {
 
 constexpr int kDmThreads = 256;
+constexpr int kChanThreads = 128;
 
 template <typename R>
 struct Super {
@@ -42,6 +47,9 @@ struct Super {
 template <typename R> struct V2;
 template <> struct V2<float> { using T = float2; };
 template <> struct V2<double> { using T = double2; };
+template <typename R> struct V16;
+template <> struct V16<float> { using T = float4; };
+template <> struct V16<double> { using T = double2; };
 
 // y = S x for one group of four amplitudes (x[l], l = 2 (row bit) + column bit)
 template <typename R>
@@ -180,6 +188,108 @@ __global__ void __launch_bounds__(kDmThreads) k_superop_inner(float *__restrict_
         super_apply<float>(S, xr, xi);
         *reinterpret_cast<float4 *>(st + 2 * base[u]) = make_float4(xr[0], xi[0], xr[1], xi[1]);
         *reinterpret_cast<float4 *>(st + 2 * (base[u] | ob)) = make_float4(xr[2], xi[2], xr[3], xi[3]);
+    }
+}
+
+// The matrix of a named channel: real, [[d0, d1], [d2, d3]] on (rho00, rho11) and
+// [[f0, f1], [f2, f3]] on (rho01, rho10); products keep the form.  A diagonal entry near 1
+// is held as its difference from 1 (the one added as x itself, bit l of
+// `one`): 1 - 2p/3 rounded to FP32 would lose or add up to 3e-8 of the trace
+// with every channel (12 qubits, 10 layers with 24 channels each, 12 circuits: the
+// trace was off by 1.3e-6 rms, always low; 1.8e-7 with the difference).
+template <typename R>
+struct Chan {
+    R m[8];
+    unsigned one;
+};
+
+template <typename R>
+__device__ __forceinline__ void chan_pair(R a, R b, R c, R d, bool one_a, bool one_d, R &x, R &y)
+{
+    const R u = a * x + (b * y + (one_a ? x : R(0)));
+    const R v = d * y + (c * x + (one_d ? y : R(0)));
+    x = u;
+    y = v;
+}
+
+// x00, x01, x10, x11: one component of the four amplitudes (row, column bit)
+template <typename R>
+__device__ __forceinline__ void chan_apply(const Chan<R> &c, R &x00, R &x01, R &x10, R &x11)
+{
+    chan_pair<R>(c.m[0], c.m[1], c.m[2], c.m[3], c.one & 1u, c.one & 2u, x00, x11);
+    chan_pair<R>(c.m[4], c.m[5], c.m[6], c.m[7], c.one & 4u, c.one & 8u, x01, x10);
+}
+
+template <typename R, int C>
+struct Chans {
+    Chan<R> c[C];
+    int q[C];                  // ascending
+};
+
+// C channels on C qubits in one pass.  A thread holds the 4^C amplitudes that
+// they mix (local index: per qubit the column bit, then the row bit) in 16-byte
+// vectors: W groups side by side over register bit 0, or, complex64 with a
+// channel on qubit 0 (W = 1), the column pair of that qubit.  complex64 is bound by
+// memory: 43 us a pass on 12 qubits (128 MiB), whatever it carries, so 6 layers with
+// two channels on every qubit took 6.2 ms one channel a pass and take 1.5 ms.
+// complex128 was bound by the FP64 units with all 16 complex entries (16 multiply-adds
+// an amplitude and channel, 4 here): those layers 111 ms, now 9.5 (135 us instead of 772
+// for one channel).  Three qubits a pass would hold 128 registers of amplitudes.
+template <typename R, int C, int W>
+__global__ void __launch_bounds__(kChanThreads) k_channels(R *__restrict__ st, uint64_t items, int n, Chans<R, C> P)
+{
+    constexpr int A = 1 << (2 * C);
+    constexpr bool kInner = sizeof(R) == 4 && W == 1;
+    constexpr int NV = kInner ? A / 2 : A;       // vectors
+    constexpr int E = 16 / sizeof(R);            // reals per vector
+    using T = typename V16<R>::T;
+    const uint64_t w = (uint64_t)blockIdx.x * kChanThreads + threadIdx.x;
+    if (w >= items) return;
+    uint64_t base = w * W;
+#pragma unroll
+    for (int i = 0; i < C; ++i) base = ((base >> P.q[i]) << (P.q[i] + 1)) | (base & ((1ull << P.q[i]) - 1ull));
+#pragma unroll
+    for (int i = 0; i < C; ++i) {
+        const int b = P.q[i] + n;
+        base = ((base >> b) << (b + 1)) | (base & ((1ull << b) - 1ull));
+    }
+    auto at = [&](int j) {
+        const int l = kInner ? 2 * j : j;
+        uint64_t off = base;
+#pragma unroll
+        for (int i = 0; i < C; ++i) {
+            if ((l >> (2 * i)) & 1) off |= 1ull << P.q[i];
+            if ((l >> (2 * i + 1)) & 1) off |= 1ull << (P.q[i] + n);
+        }
+        return reinterpret_cast<T *>(st + 2 * off);
+    };
+    R v[NV][E];
+#pragma unroll
+    for (int j = 0; j < NV; ++j) {
+        const T x = *at(j);
+        memcpy(v[j], &x, 16);
+    }
+#pragma unroll
+    for (int i = 0; i < C; ++i) {
+#pragma unroll
+        for (int l = 0; l < A; ++l) {
+            if ((l >> (2 * i)) & 3) continue;
+            const int l1 = l | (1 << (2 * i)), l2 = l | (2 << (2 * i)), l3 = l | (3 << (2 * i));
+#pragma unroll
+            for (int e = 0; e < (kInner ? 2 : E); ++e) {
+                if constexpr (kInner)
+                    chan_apply<R>(P.c[i], v[l >> 1][2 * (l & 1) + e], v[l1 >> 1][2 * (l1 & 1) + e],
+                                  v[l2 >> 1][2 * (l2 & 1) + e], v[l3 >> 1][2 * (l3 & 1) + e]);
+                else
+                    chan_apply<R>(P.c[i], v[l][e], v[l1][e], v[l2][e], v[l3][e]);
+            }
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < NV; ++j) {
+        T x;
+        memcpy(&x, v[j], 16);
+        *at(j) = x;
     }
 }
 
@@ -344,6 +454,64 @@ int launch_superop(qsim_state *s, int t, const double *kraus, int n_kraus)
     return launch_end(s, "channel");
 }
 
+// a named channel's matrix as the 8 reals of Chan (before the differences are taken)
+struct ChanMatrix {
+    double m[8];
+};
+
+static ChanMatrix channel_matrix(int kind, double p)
+{
+    double kr[32], S[32];
+    const int count = channel_kraus(kind, p, kr);
+    superop_from_kraus(kr, count, S);
+    auto re = [&](int l, int k) { return S[2 * (4 * l + k)]; };
+    return {{re(0, 0), re(0, 3), re(3, 0), re(3, 3), re(1, 1), re(1, 2), re(2, 1), re(2, 2)}};
+}
+
+// b after a
+static ChanMatrix channel_product(const ChanMatrix &b, const ChanMatrix &a)
+{
+    ChanMatrix r;
+    for (int h = 0; h < 8; h += 4)
+        for (int i = 0; i < 2; ++i)
+            for (int j = 0; j < 2; ++j)
+                r.m[h + 2 * i + j] = b.m[h + 2 * i] * a.m[h + j] + b.m[h + 2 * i + 1] * a.m[h + 2 + j];
+    return r;
+}
+
+template <typename R, int C, int W>
+static void launch_channels_as(qsim_state *s, const int *q, const ChanMatrix *m)
+{
+    Chans<R, C> P;
+    for (int i = 0; i < C; ++i) {
+        P.q[i] = q[i];
+        P.c[i].one = 0;
+        for (int k = 0; k < 8; ++k) {
+            double x = m[i].m[k];
+            if ((k & 3) % 3 == 0 && x > 0.5) {
+                P.c[i].one |= 1u << ((k >> 2) * 2 + ((k & 3) ? 1 : 0));
+                x -= 1.0;
+            }
+            P.c[i].m[k] = (R)x;
+        }
+    }
+    const uint64_t items = (1ull << (s->n - 2 * C)) / W;
+    k_channels<R, C, W><<<(unsigned)((items + kChanThreads - 1) / kChanThreads), kChanThreads, 0, s->stream>>>(
+        (R *)s->amps, items, s->n_sys, P);
+}
+
+// the channels of C qubits (ascending) in one pass
+template <int C>
+static int launch_channels(qsim_state *s, const int *q, const ChanMatrix *m)
+{
+    const double size = std::ldexp(1.0, s->n);
+    launch_begin(s, KC_CHANNEL, (s->dtype == SIM_C128 ? 32.0 : 16.0) * size, 8.0 * C * size);
+    if (s->dtype == SIM_C128) launch_channels_as<double, C, 1>(s, q, m);
+    else if (q[0] > 0) launch_channels_as<float, C, 2>(s, q, m);
+    else launch_channels_as<float, C, 1>(s, q, m);
+    return launch_end(s, "channel");
+}
+
 namespace {
 
 // a complex128 view of the diagonal roots, sharing s's stream and reduction
@@ -500,9 +668,9 @@ int sim_dm_apply_channel(sim_t s, int kind, double p, int target)
     if (target < 0 || target >= s->n_sys) return fail(SIM_EINVAL, "sim_dm_apply_channel: target out of range");
     if (!(p >= 0.0 && p <= 1.0)) return fail(SIM_EINVAL, "sim_dm_apply_channel: p must be in [0, 1]");
     double k[32];
-    const int m = channel_kraus(kind, p, k);
-    if (m == 0) return fail(SIM_EINVAL, "sim_dm_apply_channel: unknown channel kind");
-    return launch_superop(s, target, k, m);
+    if (channel_kraus(kind, p, k) == 0) return fail(SIM_EINVAL, "sim_dm_apply_channel: unknown channel kind");
+    const ChanMatrix x = channel_matrix(kind, p);
+    return launch_channels<1>(s, &target, &x);
 }
 
 int sim_dm_apply_circuit(sim_t s, const sim_gate *gates, size_t n_gates, const sim_plan_opts *opts)
@@ -548,9 +716,14 @@ int sim_dm_apply_circuit(sim_t s, const sim_gate *gates, size_t n_gates, const s
     // which fused block size absorbs the channels (0: none).  The fused plan
     // does; the learned plan does when its model picks one fused variant for
     // every window of the gates without their channels.
+    // Where the learned plan runs tiles, the channels take passes of their own,
+    // two qubits in each (7 / 9 qubits, 6 noisy Haar layers, complex128: 637 / 792 us
+    // against 883 / 1253 in blocks; complex64 9 / 11 qubits 412 / 884 us against 1059 / 1779).
     int absorb_k = 0;
     if (o.plan == SIM_PLAN_FUSED) {
         absorb_k = o.fuse_k ? o.fuse_k : (s->dtype == SIM_C128 ? 4 : 5);
+    } else if (o.plan == SIM_PLAN_LEARNED && s->cost_model && learned_tiles_only(s->n, s->dtype)) {
+        absorb_k = 0;
     } else if (o.plan == SIM_PLAN_LEARNED && s->dtype == SIM_C128 && s->cost_model && s->n >= 11) {
         absorb_k = 4;
         s->last_plan.assign(1, 4);
@@ -596,23 +769,46 @@ int sim_dm_apply_circuit(sim_t s, const sim_gate *gates, size_t n_gates, const s
         }
         return apply_sgates_fused(s, lowered, sup.data(), absorb_k);
     }
-    // runs of gates between channels under the plan; one pass per channel
+    // per gate: one pass per channel, in the order of the list.  Otherwise channels
+    // wait: those of one qubit are multiplied, a gate on other qubits goes
+    // before them, and one on a waiting qubit ends the run: the gates
+    // of the run under the plan, then its channels two qubits a pass (noise after
+    // every layer: n / 2 passes a layer instead of one per channel).
     std::vector<sim_gate> reg;
+    std::vector<ChanMatrix> wait((size_t)n);
+    uint64_t waiting = 0;
     auto flush = [&]() -> int {
-        if (reg.empty()) return SIM_OK;
-        const int rc = apply_plan(s, reg.data(), reg.size(), o);
+        if (!reg.empty())
+            if (int rc = apply_plan(s, reg.data(), reg.size(), o)) return rc;
         reg.clear();
-        return rc;
+        while (waiting) {
+            int q[2];
+            ChanMatrix m[2];
+            int c = 0;
+            for (; c < 2 && waiting; ++c, waiting &= waiting - 1) {
+                q[c] = __builtin_ctzll(waiting);
+                m[c] = wait[(size_t)q[c]];
+            }
+            if (int rc = c == 2 ? launch_channels<2>(s, q, m) : launch_channels<1>(s, q, m)) return rc;
+        }
+        return SIM_OK;
     };
     for (size_t k = 0; k < n_gates; ++k) {
         const sim_gate &g = gates[k];
+        const uint64_t bit = 1ull << g.target;
         if (is_channel_kind(g.kind)) {
-            if (int rc = flush()) return rc;
-            double kr[32];
-            const int m = channel_kraus(g.kind - SIM_GATE_CH_DEPOLARIZING, g.params[0], kr);
-            if (int rc = launch_superop(s, g.target, kr, m)) return rc;
+            const ChanMatrix x = channel_matrix(g.kind - SIM_GATE_CH_DEPOLARIZING, g.params[0]);
+            wait[(size_t)g.target] = (waiting & bit) ? channel_product(x, wait[(size_t)g.target]) : x;
+            waiting |= bit;
+            if (o.plan == SIM_PLAN_PER_GATE)
+                if (int rc = flush()) return rc;
             continue;
         }
+        uint64_t qubits = bit;
+        if (g.kind == SIM_GATE_SWAP) qubits |= 1ull << g.target2;
+        for (int c = 0; c < g.n_controls; ++c) qubits |= 1ull << g.controls[c];
+        if (qubits & waiting)
+            if (int rc = flush()) return rc;
         sim_gate two[2];
         lower_pair(g, two);
         reg.push_back(two[0]);
