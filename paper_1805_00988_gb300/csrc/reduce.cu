@@ -581,25 +581,6 @@ struct SubGeo {
 };
 
 
-// FP64 |a|^2 of the apl amplitudes of lane `lane` in sub-block `j` (zeros for
-// idle lanes and unused slots), loads first
-template <typename R>
-__device__ __forceinline__ void lane_squares(const R *st, uint64_t base, const SubGeo &g, uint32_t j, int lane,
-                                             double p[8])
-{
-    using T = typename Amp<R>::T;
-    const T *a = reinterpret_cast<const T *>(st) + base + (uint64_t)j * g.sub + (uint64_t)lane * g.apl;
-    T x[8];
-#pragma unroll
-    for (int e = 0; e < 8; ++e)
-        if ((uint32_t)lane < g.lanes && (uint32_t)e < g.apl) x[e] = a[e];
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {
-        p[e] = 0.0;
-        if ((uint32_t)lane < g.lanes && (uint32_t)e < g.apl) acc_sq<R>(p[e], x[e].x, x[e].y);
-    }
-}
-
 // warp inclusive scan of lanes 0..31, fixed order (shfl_up doubling)
 __device__ __forceinline__ double warp_incl_scan(double x, int lane)
 {
@@ -615,9 +596,10 @@ __device__ __forceinline__ double warp_incl_scan(double x, int lane)
 // sub-block each (4 per warp, 32 per CTA): lane g of a group accumulates a
 // contiguous eighth of the sub-block (complex64 full sub-blocks: compensated
 // FP32 squares carried into FP64 every 8 amplitudes; otherwise two FP64 FMAs
-// per amplitude), and a 3-step xor tree inside the group gives the sub-sum.
-// Warp 0 then scans the block's sub-sums (warp_incl_scan) and the block sum is
-// the scan's last element -- k_resolve repeats that scan bit for bit.
+// per amplitude), written to eighth[] where that is not null, and a 3-step xor
+// tree inside the group gives the sub-sum.  Warp 0 then scans the block's
+// sub-sums (warp_incl_scan); the inclusive scan goes to cum[], its last element
+// is the block sum.
 // kZ (complex64 full sub-blocks only): the same pass also forms the block's
 // <sum Z> partial as k_expz32 does (each 16-amplitude chunk's squares binned
 // by the popcount of the local index, weighted by n - 2 popcount, one
@@ -625,8 +607,8 @@ __device__ __forceinline__ double warp_incl_scan(double x, int lane)
 // 0, the pair layout k_final_sum reads).  The sub-sums are computed exactly as
 // without it.
 template <typename R, bool kZ = false>
-__global__ void __launch_bounds__(256) k_sub_sums(const R *__restrict__ st, uint64_t bs, double *__restrict__ sub,
-                                                  double *__restrict__ bsum, int n = 0,
+__global__ void __launch_bounds__(256) k_sub_sums(const R *__restrict__ st, uint64_t bs, double *__restrict__ cum,
+                                                  double *__restrict__ bsum, double *__restrict__ eighth, int n = 0,
                                                   double *__restrict__ zpart = nullptr)
 {
     using T = typename Amp<R>::T;
@@ -702,12 +684,10 @@ __global__ void __launch_bounds__(256) k_sub_sums(const R *__restrict__ st, uint
             }
         }
     }
+    if (eighth && j < g.nsub) eighth[((uint64_t)blockIdx.x * g.nsub + j) * 8 + gl] = t;
 #pragma unroll
     for (int o = 4; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-    if (gl == 0 && j < g.nsub) {
-        ss[j] = t;
-        sub[(uint64_t)blockIdx.x * g.nsub + j] = t;
-    }
+    if (gl == 0 && j < g.nsub) ss[j] = t;
     if constexpr (kZ) {
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
@@ -716,6 +696,7 @@ __global__ void __launch_bounds__(256) k_sub_sums(const R *__restrict__ st, uint
     __syncthreads();
     if (warp == 0) {
         const double c = warp_incl_scan(((uint32_t)lane < g.nsub) ? ss[lane] : 0.0, lane);
+        if ((uint32_t)lane < g.nsub) cum[(uint64_t)blockIdx.x * g.nsub + lane] = c;
         if ((uint32_t)lane == g.nsub - 1) bsum[blockIdx.x] = c;
     }
     if constexpr (kZ) {
@@ -763,7 +744,8 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_exclusive(const T *__rest
 // chunks of kScanChunk values, four contiguous values per thread.  Pass 1
 // writes each chunk's total, the one-CTA scan above turns the totals into
 // chunk offsets (and the grand total), pass 2 repeats the chunk's local scan
-// (the same operations, so the same bits) and adds the chunk's offset.
+// (the same operations, so the same bits) and adds the chunk's offset, writing
+// each value's exclusive and inclusive sum.
 constexpr int kScanChunk = 1024;
 
 template <typename T>
@@ -801,7 +783,8 @@ __global__ void __launch_bounds__(256) k_scan_chunk_sums(const T *__restrict__ i
 
 template <typename T>
 __global__ void __launch_bounds__(256) k_scan_chunk_out(const T *__restrict__ in, uint64_t nb,
-                                                        const T *__restrict__ cexcl, T *__restrict__ out)
+                                                        const T *__restrict__ cexcl, T *__restrict__ out,
+                                                        T *__restrict__ incl)
 {
     __shared__ T sh[256];
     T v[4], total;
@@ -811,47 +794,23 @@ __global__ void __launch_bounds__(256) k_scan_chunk_out(const T *__restrict__ in
     for (int e = 0; e < 4; ++e) {
         if (lo + e < nb) out[lo + e] = run;
         run += v[e];
+        if (lo + e < nb) incl[lo + e] = run;
     }
 }
 
-// shot s -> block: smallest b with bexcl[b] + bsum[b] > u_s * total; none ->
-// the last block with a non-zero sum.
-__global__ void k_locate(uint64_t shots, uint64_t seed, const double *__restrict__ bexcl,
-                         const double *__restrict__ bsum, uint64_t nb, const double *__restrict__ total,
-                         uint32_t *__restrict__ shot_blk, uint32_t *__restrict__ counts, uint64_t last_nz_blk)
+// last block with a non-zero sum (0: none), 1024 at a time from the end
+__global__ void __launch_bounds__(1024) k_last_nonzero(const double *__restrict__ bsum, uint64_t nb,
+                                                       uint64_t *__restrict__ out)
 {
-    const double tot = *total;
-    for (uint64_t s = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; s < shots;
-         s += (uint64_t)gridDim.x * blockDim.x) {
-        const double t = unif(seed, s) * tot;
-        uint64_t lo = 0, hi = nb;
-        while (lo < hi) {
-            const uint64_t mid = (lo + hi) >> 1;
-            if (bexcl[mid] + bsum[mid] > t) hi = mid; else lo = mid + 1;
+    for (uint64_t end = nb;; end -= 1024) {
+        const uint64_t i = end - 1 - threadIdx.x;
+        const bool nz = threadIdx.x < end && bsum[i] > 0.0;
+        if (__syncthreads_or(nz) || end <= 1024) {
+            if (threadIdx.x == 0) *out = 0;
+            __syncthreads();
+            if (nz) atomicMax((unsigned long long *)out, (unsigned long long)i);
+            return;
         }
-        const uint32_t b = (uint32_t)((lo < nb) ? lo : last_nz_blk);
-        shot_blk[s] = b;
-        atomicAdd(&counts[b], 1u);
-    }
-}
-
-// last block with a non-zero sum (single thread; nb scanned backwards)
-__global__ void k_last_nonzero(const double *__restrict__ bsum, uint64_t nb, uint64_t *__restrict__ out)
-{
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        uint64_t b = nb;
-        while (b > 0 && !(bsum[b - 1] > 0.0)) --b;
-        *out = (b > 0) ? b - 1 : 0;
-    }
-}
-
-__global__ void k_scatter(uint64_t shots, const uint32_t *__restrict__ shot_blk, uint32_t *__restrict__ cursor,
-                          uint32_t *__restrict__ order)
-{
-    for (uint64_t s = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; s < shots;
-         s += (uint64_t)gridDim.x * blockDim.x) {
-        const uint32_t pos = atomicAdd(&cursor[shot_blk[s]], 1u);
-        order[pos] = (uint32_t)s;
     }
 }
 
@@ -872,164 +831,267 @@ __device__ __forceinline__ void df_add(float &hi, float &lo, float th, float tl)
     lo = __fadd_rn(__fadd_rn(lo, tl), err);
 }
 
-// complex64, full sub-blocks (8 amplitudes per lane): lane `lane`'s part of
-// the in-sub-block search.  The lane's prefix is kept as compensated FP32
-// partial sums of its squares rescaled by a power of two (2^-sh, from the
-// lane's largest component).  The lanes' totals are brought to one scale (the
-// warp's largest sh) by exact powers of two and scanned across the warp as
-// FP32 pairs (TwoSum), so the only FP64 work per shot is the target t - pre
-// in that scale: this GPU's FP64 pipe runs at a small fraction of its FP32
-// rate, and an FP64 warp scan per shot made the search FP64-bound.  The
-// target relative to the lane's start, rescaled back to the lane's units, is
-// compared with each partial sum as a float pair.  An amplitude that is
-// exactly zero leaves the prefix unchanged and is never the first crossing.
-// first = the first crossing in the lane (-1: none), last_nz = the last
-// amplitude with non-zero probability (-1: none).  All 32 lanes call it.
-__device__ __forceinline__ void lane_locate32(const float *st, uint64_t base, uint32_t j, int lane, double pre,
-                                              double t, int &first, int &last_nz)
+// A non-negative finite double orders like its bits as a signed integer; a
+// negative one has negative bits, below all of them.  So a > b for a >= 0
+// takes two integer instructions instead of one on the FP64 pipe, which
+// issues one warp instruction every 16 cycles per SM.
+__device__ __forceinline__ bool above(double a, double b)
 {
-    const float4 *a4 =
-        reinterpret_cast<const float4 *>(st) + (base + (uint64_t)j * (1u << kSubLog) + (uint64_t)lane * 8) / 2;
-    float4 x[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) x[u] = a4[u];
-    float m = 0.f;
-#pragma unroll
-    for (int u = 0; u < 4; ++u) m = absmax4(m, x[u]);
-    const Pow2 pw = pow2_for(m);
-    float cs[8], ce[8];
-    bool nz[8];
+    return __double_as_longlong(a) > __double_as_longlong(b);
+}
+
+// a shot's target relative to its sub-block: (hi + lo) 2^e, |hi| in [1, 2]
+struct Target {
+    float hi, lo;
+    int e;
+};
+
+__device__ __forceinline__ Target split_target(double d)
+{
+    const uint64_t b = (uint64_t)__double_as_longlong(d);
+    const int f = (int)((b >> 52) & 0x7ffu);
+    if (f == 0) return {0.f, 0.f, 0};
+    const double m = __longlong_as_double((long long)((b & 0x800fffffffffffffull) | (1023ull << 52)));
+    const float hi = __double2float_rn(m);
+    return {hi, __double2float_rn(m - (double)hi), f - 1023};
+}
+
+// complex64: the first of the 32 amplitudes of an eighth (four in each of
+// eight lanes, gl = lane within the group) whose prefix exceeds the target.
+// The lane's prefix is kept as compensated FP32 partial sums of its squares rescaled
+// by a power of two (2^-sh, from the lane's largest component).  The lanes' totals are
+// brought to one scale (the group's largest sh) by exact powers of two and
+// scanned across the group as FP32 pairs (TwoSum).  The target, brought to
+// that scale, relative to the lane's start and rescaled back to the lane's
+// units, is compared with each partial sum as a float pair.  An amplitude that
+// is exactly zero leaves the prefix unchanged and is never the first
+// crossing.  Returns the first crossing in the lane (-1: none).
+__device__ __forceinline__ int lane_locate(const float4 x[2], int gl, const Target &tg)
+{
+    const Pow2 pw = pow2_for(absmax4(absmax4(0.f, x[0]), x[1]));
+    float cs[4], ce[4];
     Sq32 A;
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
+    for (int u = 0; u < 2; ++u) {
         const float4 y = scale4(x[u], pw.scale);
         A.add_sq(y.x); A.add_sq(y.y);
         cs[2 * u] = A.s; ce[2 * u] = A.e;
-        nz[2 * u] = x[u].x != 0.f || x[u].y != 0.f;
         A.add_sq(y.z); A.add_sq(y.w);
         cs[2 * u + 1] = A.s; ce[2 * u + 1] = A.e;
-        nz[2 * u + 1] = x[u].z != 0.f || x[u].w != 0.f;
     }
-    // the lane's total in the warp's common units 2^shm (shm >= pw.sh)
-    const int shm = __reduce_max_sync(0xffffffffu, pw.sh);
+    // the lane's total in the group's common units 2^shm (shm >= pw.sh)
+    int shm = pw.sh;
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) shm = max(shm, __shfl_xor_sync(0xffffffffu, shm, o));
     const float down = pow2f(pw.sh - shm);
     float ih = __fmul_rn(A.s, down), il = __fmul_rn(A.e, down);
-    // inclusive warp scan of the pairs, then each lane's start = the previous
-    // lane's inclusive sum
+    // inclusive scan of the pairs over the group, then each lane's start = the
+    // previous lane's inclusive sum
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const float yh = __shfl_up_sync(0xffffffffu, ih, o);
-        const float yl = __shfl_up_sync(0xffffffffu, il, o);
-        if (lane >= o) df_add(ih, il, yh, yl);
+    for (int o = 1; o < 8; o <<= 1) {
+        const float yh = __shfl_up_sync(0xffffffffu, ih, o, 8);
+        const float yl = __shfl_up_sync(0xffffffffu, il, o, 8);
+        if (gl >= o) df_add(ih, il, yh, yl);
     }
-    float sh0 = __shfl_up_sync(0xffffffffu, ih, 1), sl0 = __shfl_up_sync(0xffffffffu, il, 1);
-    if (lane == 0) { sh0 = 0.f; sl0 = 0.f; }
-    // target relative to the sub-block start in common units (FP64, then a
-    // float pair), minus the lane's start, back in the lane's units
-    double Tc = (t - pre) * __longlong_as_double((long long)((uint64_t)(1023 - shm) << 52));
-    Tc = fmin(fmax(Tc, -0x1p100), 0x1p100);
-    const float th = __double2float_rn(Tc);
-    const float tl = __double2float_rn(Tc - (double)th);
-    float rh = th, rl = tl;
+    float sh0 = __shfl_up_sync(0xffffffffu, ih, 1, 8), sl0 = __shfl_up_sync(0xffffffffu, il, 1, 8);
+    if (gl == 0) { sh0 = 0.f; sl0 = 0.f; }
+    // the target in common units (beyond 2^100: past every sum), minus the
+    // lane's start, back in the lane's units
+    const float unit = pow2f(min(tg.e - shm, 100));
+    float rh = __fmul_rn(tg.hi, unit), rl = __fmul_rn(tg.lo, unit);
     df_add(rh, rl, -sh0, -sl0);
     const float up = pow2f(shm - pw.sh);
     const bool far = shm - pw.sh > 127;            // the lane is negligible next to the largest
     rh = far ? (rh > 0.f ? INFINITY : -INFINITY) : __fmul_rn(rh, up);
     rl = far ? 0.f : __fmul_rn(rl, up);
-    first = -1;
-    last_nz = -1;
+    int first = -1;
 #pragma unroll
-    for (int e = 7; e >= 0; --e) {
-        if (nz[e] && __fadd_rn(__fsub_rn(cs[e], rh), __fsub_rn(ce[e], rl)) > 0.f) first = e;
-        if (last_nz < 0 && nz[e]) last_nz = e;
+    for (int e = 3; e >= 0; --e) {
+        const float4 &v = x[e >> 1];
+        const bool nz = (e & 1) ? (v.z != 0.f || v.w != 0.f) : (v.x != 0.f || v.y != 0.f);
+        if (nz && __fadd_rn(__fsub_rn(cs[e], rh), __fsub_rn(ce[e], rl)) > 0.f) first = e;
+    }
+    return first;
+}
+
+// complex128: the same in FP64
+__device__ __forceinline__ int lane_locate(const double2 x[4], int gl, double target)
+{
+    double c[4], run = 0.0;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        acc_sq<double>(run, x[e].x, x[e].y);
+        c[e] = run;
+    }
+    double incl = run;
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) {
+        const double y = __shfl_up_sync(0xffffffffu, incl, o, 8);
+        if (gl >= o) incl += y;
+    }
+    const double r = target - (incl - run);
+    int first = -1;
+#pragma unroll
+    for (int e = 3; e >= 0; --e)
+        if (above(c[e], r) && above(c[e], e ? c[e - 1] : 0.0)) first = e;
+    return first;
+}
+
+// Shots of a register of at least 2^8 amplitudes.  Shot s takes t = u_s total
+// and the first index whose prefix sum of |a|^2 exceeds t, found level by level:
+// the block (bexcl, bincl), the sub-block (cum, inclusive within the block), the
+// eighth of it, the amplitude.  Where rounding leaves no crossing (t within an ulp of a
+// boundary), the last one with non-zero probability is taken.
+//
+// A lane looks up the first three levels of its own shot; then eight
+// lanes read the 32 amplitudes of a shot's eighth, four shots of the warp at a time.
+// The FP64 pipe (one warp instruction every 16 cycles per SM) is kept to what a lane
+// needs for its shot.  When shots were sorted by block and a warp searched the
+// 256 amplitudes of one sub-block per shot (14 FP64 instructions a shot, 480 in all),
+// the sampling kernels took for a million shots 1.28 ms at 20 qubits (0.35 of it
+// sorting) and 1.61 at 28, complex64, and 4.2 ms at 27, complex128; now 0.14, 0.68
+// (0.55 the pass over the state) and 0.74.  The reads are as random as the shots
+// either way, 256 bytes (512) per shot.
+template <typename R>
+__global__ void __launch_bounds__(256) k_shots(const R *__restrict__ st, uint32_t nsub, uint64_t seed,
+                                               const double *__restrict__ bexcl, const double *__restrict__ bincl,
+                                               uint64_t nb, const double *__restrict__ total,
+                                               const uint64_t *__restrict__ last, const double *__restrict__ cum,
+                                               const double *__restrict__ eighth, uint64_t shots,
+                                               uint64_t *__restrict__ out)
+{
+    using V = typename std::conditional<sizeof(R) == 4, float4, double2>::type;
+    constexpr int NV = sizeof(R) == 4 ? 2 : 4;         // 16-byte vectors of a lane's four amplitudes
+    const double tot = *total;
+    if (!(tot > 0.0)) return;
+    const int lane = threadIdx.x & 31, gr = lane >> 3, gl = lane & 7;
+    const uint64_t step = (uint64_t)gridDim.x * blockDim.x;
+    for (uint64_t c0 = (uint64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); c0 < shots; c0 += step) {
+        const uint64_t s = min(c0 + (uint64_t)lane, shots - 1);
+        const double t = unif(seed, s) * tot;
+        uint64_t lo = 0, hi = nb;
+        while (lo < hi) {
+            const uint64_t mid = (lo + hi) >> 1;
+            if (above(bincl[mid], t)) hi = mid; else lo = mid + 1;
+        }
+        const uint64_t b = lo < nb ? lo : *last;
+        const double be = bexcl[b];
+        const double *P = cum + b * nsub;
+        uint32_t j = 0, je = nsub;
+        while (j < je) {
+            const uint32_t mid = (j + je) >> 1;
+            if (above(be + P[mid], t)) je = mid; else j = mid + 1;
+        }
+        if (j == nsub)
+            for (--j; j > 0 && !(P[j] > P[j - 1]);) --j;
+        const double d = t - (be + (j > 0 ? P[j - 1] : 0.0));
+        const uint64_t q = b * nsub + j;
+        // the last eighth that is not empty and starts at or before the target
+        const double2 *e2 = reinterpret_cast<const double2 *>(eighth + 8 * q);
+        double ev[8], acc = 0.0, gp = 0.0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const double2 y = e2[k];
+            ev[2 * k] = y.x;
+            ev[2 * k + 1] = y.y;
+        }
+        int g = -1;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            if (above(ev[k], 0.0) && (g < 0 || !above(acc, d))) {
+                g = k;
+                gp = acc;
+            }
+            if (k < 7) acc += ev[k];
+        }
+        const uint32_t part = (uint32_t)(q * 8) + (uint32_t)max(g, 0);   // 32 amplitudes each
+        const double rel = d - gp;
+        Target tl = {0.f, 0.f, 0};
+        if constexpr (sizeof(R) == 4) tl = split_target(rel);
+        const V *av = reinterpret_cast<const V *>(st) + gl * NV;
+        V nx[NV];
+        {
+            const uint64_t p = __shfl_sync(0xffffffffu, part, gr);
+#pragma unroll
+            for (int u = 0; u < NV; ++u) nx[u] = av[p * (8 * NV) + u];
+        }
+        uint32_t idx = 0;
+#pragma unroll 1
+        for (int it = 0; it < 8; ++it) {
+            const int i = it * 4 + gr;
+            V x[NV];
+#pragma unroll
+            for (int u = 0; u < NV; ++u) x[u] = nx[u];
+            const uint64_t p = __shfl_sync(0xffffffffu, part, min(i + 4, 28 + gr));
+#pragma unroll
+            for (int u = 0; u < NV; ++u) nx[u] = av[p * (8 * NV) + u];
+            int hit;
+            if constexpr (sizeof(R) == 4)
+                hit = lane_locate(x, gl, Target{__shfl_sync(0xffffffffu, tl.hi, i), __shfl_sync(0xffffffffu, tl.lo, i),
+                                                __shfl_sync(0xffffffffu, tl.e, i)});
+            else
+                hit = lane_locate(x, gl, __shfl_sync(0xffffffffu, rel, i));
+            uint32_t fl = (__ballot_sync(0xffffffffu, hit >= 0) >> (8 * gr)) & 0xffu;
+            if (__any_sync(0xffffffffu, fl == 0)) {        // no crossing: the last one that is not zero
+                int nz = -1;
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    if constexpr (sizeof(R) == 4) {
+                        const float4 &v = x[e >> 1];
+                        if ((e & 1) ? (v.z != 0.f || v.w != 0.f) : (v.x != 0.f || v.y != 0.f)) nz = e;
+                    } else {
+                        double p2 = 0.0;
+                        acc_sq<double>(p2, x[e].x, x[e].y);
+                        if (p2 > 0.0) nz = e;
+                    }
+                }
+                const uint32_t nl = (__ballot_sync(0xffffffffu, nz >= 0) >> (8 * gr)) & 0xffu;
+                if (fl == 0) {
+                    hit = max(nz, 0);
+                    fl = nl ? 1u << (31 - __clz(nl)) : 1u;
+                }
+            }
+            const int L = __ffs(fl) - 1;
+            const uint32_t found = (uint32_t)(4 * L + __shfl_sync(0xffffffffu, hit, 8 * gr + L));
+            const uint32_t mine = __shfl_sync(0xffffffffu, found, 8 * (lane & 3));
+            if ((lane >> 2) == it) idx = mine;
+        }
+        if (c0 + (uint64_t)lane < shots) out[s] = (uint64_t)part * 32 + idx;
     }
 }
 
-// Persistent warps over the shots in block order (the counting sort puts the
-// shots of one block next to each other): warp w takes shots
-// [w * per, (w + 1) * per) of `order`.  On entering a new block the warp
-// rebuilds that block's inclusive scan of sub-sums P (lane j holds P[j]; the
-// same operations as k_sub_sums, so the same bits) and its exclusive prefix.
-// Per shot: t = u_s * total; the sub-block is the first j with
-// bexcl + P[j] > t; the warp scans its amplitudes (lane-serial prefix, then a
-// warp scan of lane totals) and the outcome is the first index whose prefix
-// exceeds t.  Where rounding leaves no crossing (t within an ulp of a
-// boundary), the last sub-block / amplitude with non-zero probability is
-// taken.
+// the same for a register of fewer than 2^8 amplitudes: their prefix in shared
+// memory, a thread per shot
 template <typename R>
-__global__ void __launch_bounds__(256) k_resolve(const R *__restrict__ st, uint64_t bs, uint64_t seed,
-                                                 const double *__restrict__ bexcl, const double *__restrict__ total,
-                                                 const double *__restrict__ sub, const uint32_t *__restrict__ shot_blk,
-                                                 const uint32_t *__restrict__ order, uint64_t shots, uint64_t per,
-                                                 uint64_t *__restrict__ out)
+__global__ void __launch_bounds__(256) k_shots_small(const R *__restrict__ st, uint32_t N, uint64_t seed,
+                                                     const double *__restrict__ total, uint64_t shots,
+                                                     uint64_t *__restrict__ out)
 {
-    const SubGeo g(bs);
-    const int lane = threadIdx.x & 31;
-    const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const uint64_t k0 = warp * per;
-    const uint64_t k1 = min(shots, k0 + per);
+    __shared__ double pre[128];
+    __shared__ uint32_t last;
     const double tot = *total;
-    uint32_t cur = 0xFFFFFFFFu;          // block whose scan the warp holds
-    double Pl = 0.0, be = 0.0;
-    unsigned sub_nz = 0u;
-    // the shot numbers and blocks of 32 shots at a time: lane i loads those
-    // of shot c0 + i (one coalesced load and one gather for 32 shots instead
-    // of two dependent loads per shot), the loop takes them by shuffle
-    for (uint64_t c0 = k0; c0 < k1; c0 += 32) {
-        const uint64_t kl = c0 + (uint64_t)lane;
-        const uint32_t s_l = kl < k1 ? order[kl] : 0u;
-        const uint32_t b_l = kl < k1 ? shot_blk[s_l] : 0u;
-        const int cnt = (int)min((uint64_t)32, k1 - c0);
-        for (int i = 0; i < cnt; ++i) {
-            const uint32_t s = __shfl_sync(0xffffffffu, s_l, i);
-            const uint32_t blk = __shfl_sync(0xffffffffu, b_l, i);
-            if (blk != cur) {
-                cur = blk;
-                Pl = warp_incl_scan(((uint32_t)lane < g.nsub) ? sub[(uint64_t)blk * g.nsub + lane] : 0.0, lane);
-                be = bexcl[blk];
-                const double prev = __shfl_up_sync(0xffffffffu, Pl, 1);
-                const bool lane_nz = (uint32_t)lane < g.nsub && (lane == 0 ? Pl > 0.0 : Pl > prev);
-                sub_nz = __ballot_sync(0xffffffffu, lane_nz);
-            }
-            const uint64_t base = (uint64_t)blk * bs;
-            const double t = unif(seed, s) * tot;
-            const unsigned hit = __ballot_sync(0xffffffffu, (uint32_t)lane < g.nsub && be + Pl > t);
-            const uint32_t j = hit ? (uint32_t)(__ffs(hit) - 1) : (sub_nz ? (uint32_t)(31 - __clz(sub_nz)) : 0u);
-            const double pj = __shfl_sync(0xffffffffu, Pl, (int)(j > 0 ? j - 1 : 0));
-            const double pre = be + (j > 0 ? pj : 0.0);
-            int first = -1, last_nz = -1;
-            if (sizeof(R) == 4 && g.apl == 8) {
-                lane_locate32(reinterpret_cast<const float *>(st), base, j, lane, pre, t, first, last_nz);
-            } else {
-                double p[8];
-                lane_squares<R>(st, base, g, j, lane, p);
-                double c[8], run = 0.0;
-#pragma unroll
-                for (int e = 0; e < 8; ++e) {
-                    run += p[e];
-                    c[e] = run;
-                }
-                const double incl = warp_incl_scan(run, lane);
-                const double start = pre + (incl - run);
-#pragma unroll
-                for (int e = 7; e >= 0; --e) {
-                    if ((uint32_t)e < g.apl && start + c[e] > t) first = e;
-                    if (last_nz < 0 && p[e] > 0.0) last_nz = e;
-                }
-            }
-            const unsigned fl = __ballot_sync(0xffffffffu, first >= 0);
-            uint64_t idx;
-            if (fl) {
-                const int L = __ffs(fl) - 1;
-                idx = (uint64_t)L * g.apl + (uint64_t)__shfl_sync(0xffffffffu, first, L);
-            } else {
-                const unsigned nl = __ballot_sync(0xffffffffu, last_nz >= 0);
-                const int L = nl ? 31 - __clz(nl) : 0;
-                const int e = __shfl_sync(0xffffffffu, last_nz, L);
-                idx = (uint64_t)L * g.apl + (uint64_t)(e > 0 ? e : 0);
-            }
-            if (lane == 0) out[s] = base + (uint64_t)j * g.sub + idx;
+    if (!(tot > 0.0)) return;
+    if (threadIdx.x == 0) {
+        double run = 0.0;
+        last = 0;
+        for (uint32_t i = 0; i < N; ++i) {
+            double p = 0.0;
+            acc_sq<R>(p, st[2 * i], st[2 * i + 1]);
+            run += p;
+            pre[i] = run;
+            if (p > 0.0) last = i;
         }
+    }
+    __syncthreads();
+    for (uint64_t s = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; s < shots;
+         s += (uint64_t)gridDim.x * blockDim.x) {
+        const double t = unif(seed, s) * tot;
+        uint32_t lo = 0, hi = N;
+        while (lo < hi) {
+            const uint32_t mid = (lo + hi) >> 1;
+            if (above(pre[mid], t)) hi = mid; else lo = mid + 1;
+        }
+        out[s] = lo < N ? lo : last;
     }
 }
 
@@ -1042,10 +1104,10 @@ unsigned grid_for(uint64_t work, int threads, int num_sms)
     return (unsigned)g;
 }
 
-// exclusive scan of nb values into out and their total into *total, on the
-// handle's stream; cs holds 2 * ceil(nb / kScanChunk) values of scratch
+// exclusive scan of nb values into out, inclusive into incl and their total
+// into *total, on the handle's stream; cs holds 2 * ceil(nb / kScanChunk) values of scratch
 template <typename T>
-int scan_exclusive(qsim_state *s, const T *in, T *out, uint64_t nb, T *total, T *cs, const char *what)
+int scan_sums(qsim_state *s, const T *in, T *out, T *incl, uint64_t nb, T *total, T *cs, const char *what)
 {
     const uint64_t nc = (nb + kScanChunk - 1) / kScanChunk;
     launch_begin(s, KC_SAMPLE);
@@ -1055,7 +1117,7 @@ int scan_exclusive(qsim_state *s, const T *in, T *out, uint64_t nb, T *total, T 
     k_scan_exclusive<T><<<1, kScanThreads, 0, s->stream>>>(cs, cs + nc, nc, total);
     if (int rc = launch_end(s, what)) return rc;
     launch_begin(s, KC_SAMPLE);
-    k_scan_chunk_out<T><<<(unsigned)nc, 256, 0, s->stream>>>(in, nb, cs + nc, out);
+    k_scan_chunk_out<T><<<(unsigned)nc, 256, 0, s->stream>>>(in, nb, cs + nc, out, incl);
     return launch_end(s, what);
 }
 
@@ -1186,96 +1248,72 @@ int run_sample(qsim_state *s, uint64_t shots, uint64_t seed, uint64_t *out, int 
     const uint64_t bs = (s->n >= kSampleLog) ? (1ull << kSampleLog) : N;
     const uint64_t nb = N / bs;
     const SubGeo sg(bs);
-    // scratch: sub-sums (nb * nsub doubles), bsum, bexcl (nb doubles), counts, offs, cursor (nb u32),
-    //          total, last (8 B each), shot_blk, order (shots u32), out (shots u64 for host output),
-    //          chunk totals and offsets of the two scans
+    // scratch: scanned sub-sums and eighths of full sub-blocks, block sums and
+    // their scans (nb doubles each), total, last block and <sum Z>, chunk
+    // totals and offsets of the scan, shots for host output
+    const bool full = sg.sub == (1u << kSubLog);
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t o = off; off += (bytes + 255) & ~(size_t)255; return o; };
-    const size_t o_sub = take(nb * sg.nsub * 8);
-    const size_t o_bsum = take(nb * 8), o_bexcl = take(nb * 8), o_tot = take(8), o_last = take(8);
-    const size_t o_cnt = take(nb * 4), o_offs = take(nb * 4), o_cur = take(nb * 4), o_u32tot = take(8);
-    const size_t o_sblk = take(shots * 4), o_order = take(shots * 4);
+    const size_t o_cum = take(nb * sg.nsub * 8), o_eig = full ? take(nb * sg.nsub * 64) : 0;
+    const size_t o_bsum = take(nb * 8), o_bexcl = take(nb * 8), o_bincl = take(nb * 8), o_tot = take(4 * 8);
     const uint64_t nchunk = (nb + kScanChunk - 1) / kScanChunk;
-    const size_t o_cs = take(2 * nchunk * 8), o_cs32 = take(2 * nchunk * 4);
-    const size_t o_zpart = obs ? take(2 * nb * 8) : 0, o_zout = obs ? take(2 * 8) : 0;
+    const size_t o_cs = take(2 * nchunk * 8);
+    const size_t o_zpart = obs ? take(2 * nb * 8) : 0;
     const size_t o_out = out_on_device ? 0 : take(shots * 8);
     char *scratch = nullptr;
     QSIM_CUDA(cudaMallocAsync((void **)&scratch, off, s->stream));
-    double *sub = (double *)(scratch + o_sub);
+    double *cum = (double *)(scratch + o_cum), *eighth = full ? (double *)(scratch + o_eig) : nullptr;
     double *bsum = (double *)(scratch + o_bsum), *bexcl = (double *)(scratch + o_bexcl);
-    double *tot = (double *)(scratch + o_tot);
-    uint64_t *last = (uint64_t *)(scratch + o_last);
-    uint32_t *cnt = (uint32_t *)(scratch + o_cnt), *offs = (uint32_t *)(scratch + o_offs);
-    uint32_t *cur = (uint32_t *)(scratch + o_cur), *u32tot = (uint32_t *)(scratch + o_u32tot);
-    uint32_t *sblk = (uint32_t *)(scratch + o_sblk), *order = (uint32_t *)(scratch + o_order);
+    double *bincl = (double *)(scratch + o_bincl);
+    double *tot = (double *)(scratch + o_tot), *zout = tot + 2;        // zout: two values
+    uint64_t *last = (uint64_t *)(tot + 1);
     uint64_t *dout = out_on_device ? out : (uint64_t *)(scratch + o_out);
     double *cs = (double *)(scratch + o_cs);
-    uint32_t *cs32 = (uint32_t *)(scratch + o_cs32);
-    double *zpart = obs ? (double *)(scratch + o_zpart) : nullptr, *zout = obs ? (double *)(scratch + o_zout) : nullptr;
+    double *zpart = obs ? (double *)(scratch + o_zpart) : nullptr;
     int rc = SIM_OK;
     const bool c128 = s->dtype == SIM_C128;
     do {
         launch_begin(s, KC_SAMPLE, (double)s->bytes);
-        if (c128) k_sub_sums<double><<<(unsigned)nb, 256, 0, s->stream>>>((const double *)s->amps, bs, sub, bsum);
+        if (c128) k_sub_sums<double><<<(unsigned)nb, 256, 0, s->stream>>>((const double *)s->amps, bs, cum, bsum, eighth);
         else if (obs)
-            k_sub_sums<float, true><<<(unsigned)nb, 256, 0, s->stream>>>((const float *)s->amps, bs, sub, bsum, s->n,
-                                                                       zpart);
-        else k_sub_sums<float><<<(unsigned)nb, 256, 0, s->stream>>>((const float *)s->amps, bs, sub, bsum);
+            k_sub_sums<float, true><<<(unsigned)nb, 256, 0, s->stream>>>((const float *)s->amps, bs, cum, bsum, eighth,
+                                                                       s->n, zpart);
+        else k_sub_sums<float><<<(unsigned)nb, 256, 0, s->stream>>>((const float *)s->amps, bs, cum, bsum, eighth);
         if ((rc = launch_end(s, "sub-block sums"))) break;
         if (obs) {
             launch_begin(s, KC_REDUCE);
             k_final_sum<<<1, kRedThreads, 0, s->stream>>>(zpart, (int)nb, zout);
             if ((rc = launch_end(s, "<sum Z> total"))) break;
         }
-        if ((rc = scan_exclusive<double>(s, bsum, bexcl, nb, tot, cs, "block scan"))) break;
+        if ((rc = scan_sums<double>(s, bsum, bexcl, bincl, nb, tot, cs, "block scan"))) break;
         launch_begin(s, KC_SAMPLE);
-        k_last_nonzero<<<1, 32, 0, s->stream>>>(bsum, nb, last);
+        k_last_nonzero<<<1, 1024, 0, s->stream>>>(bsum, nb, last);
         if ((rc = launch_end(s, "last nonzero"))) break;
-        // the host needs the last non-zero block as a launch argument: read it
-        // together with the total (one small copy; the state stays on device)
-        double htot = 0.0, hz = 0.0;
-        uint64_t hlast = 0;
-        if (cudaMemcpyAsync(&htot, tot, 8, cudaMemcpyDeviceToHost, s->stream) != cudaSuccess ||
-            cudaMemcpyAsync(&hlast, last, 8, cudaMemcpyDeviceToHost, s->stream) != cudaSuccess ||
-            (obs && cudaMemcpyAsync(&hz, zout, 8, cudaMemcpyDeviceToHost, s->stream) != cudaSuccess) ||
+        // per shot 32 amplitudes; a zero norm writes none
+        launch_begin(s, KC_SAMPLE, (double)shots * (full ? 32.0 : 0.0) * (c128 ? 16.0 : 8.0));
+        const unsigned grid = grid_for(shots, 256, s->num_sms);
+        if (full && c128)
+            k_shots<double><<<grid, 256, 0, s->stream>>>((const double *)s->amps, sg.nsub, seed, bexcl, bincl, nb, tot,
+                                                         last, cum, eighth, shots, dout);
+        else if (full)
+            k_shots<float><<<grid, 256, 0, s->stream>>>((const float *)s->amps, sg.nsub, seed, bexcl, bincl, nb, tot,
+                                                        last, cum, eighth, shots, dout);
+        else if (c128)
+            k_shots_small<double><<<grid, 256, 0, s->stream>>>((const double *)s->amps, (uint32_t)N, seed, tot, shots,
+                                                               dout);
+        else
+            k_shots_small<float><<<grid, 256, 0, s->stream>>>((const float *)s->amps, (uint32_t)N, seed, tot, shots,
+                                                              dout);
+        if ((rc = launch_end(s, "shots"))) break;
+        double *host = s->host_red;
+        if (cudaMemcpyAsync(host, tot, (obs ? 3 : 1) * 8, cudaMemcpyDeviceToHost, s->stream) != cudaSuccess ||
             cudaStreamSynchronize(s->stream) != cudaSuccess) {
             rc = cuda_fail(cudaGetLastError(), "sample readback");
             break;
         }
-        if (norm_out) *norm_out = htot;
-        if (expz_out) *expz_out = hz;
-        if (!(htot > 0.0)) { rc = fail(SIM_EINVAL, "sim_sample: the state has zero norm"); break; }
-        if (cudaMemsetAsync(cnt, 0, nb * 4, s->stream) != cudaSuccess) { rc = cuda_fail(cudaGetLastError(), "memset"); break; }
-        launch_begin(s, KC_SAMPLE);
-        k_locate<<<grid_for(shots, 256, s->num_sms), 256, 0, s->stream>>>(shots, seed, bexcl, bsum, nb, tot, sblk,
-                                                                           cnt, hlast);
-        if ((rc = launch_end(s, "locate shots"))) break;
-        if ((rc = scan_exclusive<uint32_t>(s, cnt, offs, nb, u32tot, cs32, "bucket scan"))) break;
-        if (cudaMemcpyAsync(cur, offs, nb * 4, cudaMemcpyDeviceToDevice, s->stream) != cudaSuccess) {
-            rc = cuda_fail(cudaGetLastError(), "cursor copy");
-            break;
-        }
-        launch_begin(s, KC_SAMPLE);
-        k_scatter<<<grid_for(shots, 256, s->num_sms), 256, 0, s->stream>>>(shots, sblk, cur, order);
-        if ((rc = launch_end(s, "scatter shots"))) break;
-        // per shot: one sub-block of amplitudes; warps as many as are resident
-        launch_begin(s, KC_SAMPLE, (double)shots * sg.sub * (c128 ? 16.0 : 8.0));
-        {
-            const void *fn = c128 ? (const void *)k_resolve<double> : (const void *)k_resolve<float>;
-            int per_sm = 0;
-            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, 256, 0) != cudaSuccess || per_sm < 1)
-                per_sm = 1;
-            const uint64_t warps = (uint64_t)s->num_sms * per_sm * 8;
-            const uint64_t per = (shots + warps - 1) / warps;
-            const unsigned grid = (unsigned)((shots + per * 8 - 1) / (per * 8));
-            if (c128)
-                k_resolve<double><<<grid, 256, 0, s->stream>>>((const double *)s->amps, bs, seed, bexcl, tot, sub, sblk,
-                                                               order, shots, per, dout);
-            else
-                k_resolve<float><<<grid, 256, 0, s->stream>>>((const float *)s->amps, bs, seed, bexcl, tot, sub, sblk,
-                                                              order, shots, per, dout);
-        }
-        if ((rc = launch_end(s, "resolve shots"))) break;
+        if (norm_out) *norm_out = host[0];
+        if (expz_out) *expz_out = host[2];
+        if (!(host[0] > 0.0)) { rc = fail(SIM_EINVAL, "sim_sample: the state has zero norm"); break; }
         if (!out_on_device) {
             if (cudaMemcpyAsync(out, dout, shots * 8, cudaMemcpyDeviceToHost, s->stream) != cudaSuccess) {
                 rc = cuda_fail(cudaGetLastError(), "shots readback");
