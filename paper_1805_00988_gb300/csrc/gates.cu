@@ -132,6 +132,7 @@ struct PairArgs {
     uint64_t hi_off;       // second amplitude = base | hi_off
     int npos;              // zero bits inserted at pos[0] < pos[1] < ...
     int pos[4];
+    bool real;             // every entry of the matrix is real
 };
 
 template <typename R>
@@ -150,10 +151,38 @@ __device__ __forceinline__ uint64_t insert_zeros(uint64_t w, const PairArgs &a)
     return w;
 }
 
+// complex128: the FP64 pipe issues a warp instruction every 16 cycles per SM,
+// so a dense gate's arithmetic outlasts its traffic.  Four chained multiply-adds per
+// component (16 instructions a pair instead of the 20 that sums of two products
+// make), two if the matrix is real (H, RY): 22 qubits, H 85 -> 35 us, Haar + CZ layers
+// 60 -> 47 us a gate.
+__device__ __forceinline__ void dense64(double &lr, double &li, double &hr, double &hi, const Coef<double> &c, bool real)
+{
+    double nlr = c.ar * lr, nli = c.ar * li, nhr = c.cr * lr, nhi = c.cr * li;
+    if (!real) {
+        nlr = fma(-c.ai, li, nlr);
+        nli = fma(c.ai, lr, nli);
+        nhr = fma(-c.ci, li, nhr);
+        nhi = fma(c.ci, lr, nhi);
+        nlr = fma(-c.bi, hi, nlr);
+        nli = fma(c.bi, hr, nli);
+        nhr = fma(-c.di, hi, nhr);
+        nhi = fma(c.di, hr, nhi);
+    }
+    lr = fma(c.br, hr, nlr);
+    li = fma(c.br, hi, nli);
+    hr = fma(c.dr, hr, nhr);
+    hi = fma(c.dr, hi, nhi);
+}
+
 // the update of one amplitude pair (lo = v_a, hi = v_b)
 template <int OP, typename R>
-__device__ __forceinline__ void pair_update(R &lr, R &li, R &hr, R &hi, const Coef<R> &c)
+__device__ __forceinline__ void pair_update(R &lr, R &li, R &hr, R &hi, const Coef<R> &c, bool real = false)
 {
+    if constexpr (OP == OP_DENSE && sizeof(R) == 8) {
+        dense64(lr, li, hr, hi, c, real);
+        return;
+    }
     if (OP == OP_DENSE) {
         const R nlr = c.ar * lr - c.ai * li + (c.br * hr - c.bi * hi);
         const R nli = c.ar * li + c.ai * lr + (c.br * hi + c.bi * hr);
@@ -205,8 +234,13 @@ constexpr int kThreads = 256;
 //    work on 16 SMs.
 // 14 qubits: 5.2 -> 1.9 us a gate complex128, 4.1 -> 1.9 complex64; 24 qubits
 // still gain the latency (31.2 -> 28.8 us).
+// complex128 takes the small blocks further up: a kernel launched early gets
+// the SMs that the one before left free, so a few big blocks spread unevenly, and
+// the FP64 pipe of the fullest SM decides (18 qubits, U3 + CNOT ladder: 10.9 us a gate
+// with 512-pair blocks, 5.5 with 64; 20 qubits 12.6 and 11.3; from 21 on, and for
+// controlled and diagonal gates from 20 on, the big ones win).
 constexpr int kSmallThreads = 64;
-constexpr uint64_t kSpread = 152;
+constexpr uint64_t kSpread = 152, kSpread64 = 608, kSpreadDense64 = 1216;
 
 __device__ __forceinline__ void pdl_enter()
 {
@@ -263,7 +297,7 @@ __global__ void __launch_bounds__(kThreads) k_pair_split(R *__restrict__ st, Pai
             stv<R, VEC>(st, base[u] | a.hi_off, h);
         } else {
             V l = (OP != OP_DIAG_HI) ? lo[u] : V{}, h = hi[u];
-            pair_update<OP, R>(l.x, l.y, h.x, h.y, c);
+            pair_update<OP, R>(l.x, l.y, h.x, h.y, c, a.real);
             if (OP != OP_DIAG_HI) stv<R, VEC>(st, base[u] | a.lo_off, l);
             stv<R, VEC>(st, base[u] | a.hi_off, h);
         }
@@ -310,7 +344,7 @@ template <typename R, int VEC, int OP, int U>
 void go_split(qsim_state *s, const PairArgs &a, const Coef<R> &c)
 {
     const uint64_t per = (uint64_t)kThreads * U, blocks = (a.n_items + per - 1) / per;
-    if (blocks >= kSpread)
+    if (blocks >= (sizeof(R) == 4 ? kSpread : OP == OP_DENSE ? kSpreadDense64 : kSpread64))
         launch_pdl(s->stream, k_pair_split<R, VEC, OP, U>, blocks, kThreads, (R *)s->amps, a, c);
     else
         launch_pdl(s->stream, k_pair_split<R, VEC, OP, 1>, (a.n_items + kSmallThreads - 1) / kSmallThreads,
@@ -408,6 +442,7 @@ static int launch_pair_impl(qsim_state *s, const PairGate &g, uint64_t cm)
         a.lo_off = 0;
         a.hi_off = 1ull << g.target;
     }
+    a.real = g.m[1] == 0.0 && g.m[3] == 0.0 && g.m[5] == 0.0 && g.m[7] == 0.0;
     const uint64_t bases = 1ull << (s->n - np);
     // amplitudes the gate must change: 2 per base (1 for a phase on |1>), read + written
     const double amp = (s->dtype == SIM_C128) ? 16.0 : 8.0;
