@@ -30,6 +30,7 @@
 #include <cstring>
 #include <vector>
 
+#include "f32x2.cuh"
 #include "tile.cuh"
 
 namespace qsim {
@@ -91,33 +92,6 @@ template <> struct V2<double> { using T = double2; };
 // were carried separately from one operation to the next, and the moves that
 // paired them up again were a third of all instructions.  complex128 keeps
 // plain doubles.
-typedef unsigned long long pack2;
-__device__ __forceinline__ pack2 pk(float x, float y)
-{
-    pack2 v;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(x), "f"(y));
-    return v;
-}
-__device__ __forceinline__ float2 unpk(pack2 v)
-{
-    float2 r;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-    return r;
-}
-__device__ __forceinline__ pack2 fma2(pack2 a, pack2 b, pack2 c)
-{
-    pack2 d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-__device__ __forceinline__ pack2 mul2(pack2 a, pack2 b)
-{
-    pack2 d;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ pack2 dup(float x) { return pk(x, x); }
-
 template <typename R, int RA> struct Amps;
 template <int RA> struct Amps<float, RA> {
     pack2 r[RA / 2], i[RA / 2];
