@@ -112,3 +112,18 @@ def test_probabilities_and_collapse_vectors(sim, dt, n):
         assert abs(pm - p64[keep].sum()) <= 1e-6 and np.all(got[~keep] == 0)
         assert np.all(np.abs(got - want) <= 4 * eps * np.abs(want) + 1e-45)
     st.close()
+
+
+def test_measured_halves_by_qubit(sim):
+    """23 qubits: batches of 8 strided vectors, qubits inside a vector, below the
+    stride, within the batch's span and above it.  Compensated sums: 1e-12 of the total."""
+    n = 23
+    psi = C.random_state(n, seed=n).astype(np.complex64)
+    p = psi.real.astype(np.float64) ** 2 + psi.imag.astype(np.float64) ** 2
+    st = sim.State(n, "c64")
+    for q in (0, 1, 8, 9, 10, 11, 12, 13, n - 1):
+        st.load(psi)
+        m, pm = sim.sim_measure(st.h, q, 3)
+        half = p.reshape(-1, 2, 1 << q)[:, m].sum()
+        assert abs(pm - half / p.sum()) <= 1e-12
+    st.close()
