@@ -22,7 +22,15 @@
 //
 // Precision: two roundings per gate and amplitude instead of four, plus one
 // complex multiply per merged diagonal; tables and shears are formed in FP64
-// on the host and rounded once.  Pending scale factors stay within 2^-8..2^8.
+// on the host and rounded once.
+//
+// Range.  The amplitudes in memory are the state without the pending factors,
+// so those must stay where FP32 tables and FP32 amplitudes hold them: the
+// common factor is applied when it leaves 2^-8..2^8; a rotation leaves a factor
+// of modulus 1/4..4 on its qubit, which the next one takes; pairs have modulus
+// one; and a gate whose own factors are not of modulus one (a contraction, say) is
+// kept aside only while all moduli pending stay within kPoolBits bits together,
+// otherwise applied where it stands.
 #pragma once
 
 #include <cmath>
@@ -1047,6 +1055,11 @@ inline bool pool_factor(cplx f)
     const double a = std::abs(f);
     return a > 1e-6 && a < 1e6;
 }
+// modulus one to FP32 rounding of the entries: such factors may pile up without
+// leaving the range (a million of them by less than two bits)
+inline bool unit_factor(cplx f) { return std::abs(std::norm(f) - 1.0) <= 2e-6; }
+// as far as the common factor may go
+constexpr double kPoolBits = 8.0;
 
 // One operation before packing; the first five kinds are packed into groups.
 enum IrKind { IR_Z = 0, IR_DIAG, IR_SHEARS, IR_FLUSH, IR_LAYOUT, IR_RAMP, IR_XCH, IR_PH, IR_CSHEARS, IR_PERM };
@@ -1198,7 +1211,7 @@ public:
             swap_places(g.target, g.target2);
             return;
         }
-        if (nc == 0 && g.op == OP_ANTIDIAG && pool_factor(B) && pool_factor(C)) {
+        if (nc == 0 && g.op == OP_ANTIDIAG && takes(C, B)) {
             pool.g *= C;
             pool.y[g.target] *= B / C;       // X diag(C, B)
             relabel(g.target);
@@ -1267,6 +1280,16 @@ private:
         }
     }
     bool flipped(int q) const { return (flip_ >> q) & 1ull; }
+    // whether the pool may take a gate's factors a and d (of a qubit's 0 and 1)
+    bool takes(cplx a, cplx d) const
+    {
+        if (!pool_factor(a) || !pool_factor(d)) return false;
+        if (unit_factor(a) && unit_factor(d)) return true;
+        auto bits = [](cplx f) { return unit_factor(f) ? 0.0 : std::abs(std::log2(std::abs(f))); };
+        double t = bits(a) + bits(d) + bits(pool.g);
+        for (const cplx &f : pool.y) t += bits(f);
+        return t <= kPoolBits;
+    }
     // logical value of qubit q (a register bit) in register k
     int bit_of(int q, int k) const { return ((k >> reg_[(size_t)q]) & 1) ^ (flipped(q) ? 1 : 0); }
 
@@ -1615,6 +1638,7 @@ private:
         const cplx f0 = f ? P1 : P0, f1 = f ? P0 : P1;
         pool.g *= f0;
         pool.y[(size_t)x] = f1 / f0;
+        if (std::norm(p) + std::norm(q) < 0.5 || std::norm(p) + std::norm(q) > 8.0) close_group();   // a scaled matrix: its scale does not wait
         return true;
     }
 
@@ -1657,7 +1681,10 @@ private:
         }
         const cplx f0 = fl ? P1 : P0, f1 = fl ? P0 : P1;
         pool.g *= f0;
-        pool.y[(size_t)x] = f1 / f0;
+        const cplx left = f1 / f0;
+        if (std::abs(left) < 0.5 || std::abs(left) > 2.0) tab_single(x, left);   // not kept aside
+        else pool.y[(size_t)x] = left;
+        close_group();
         return true;
     }
 
@@ -1754,7 +1781,7 @@ private:
         const int nc = __builtin_popcountll(g.ctrl);
         const cplx a = (g.op == OP_DIAG) ? cplx(g.m[0], g.m[1]) : cplx(1.0), d(g.m[6], g.m[7]);
         const int x = g.target;
-        if (nc <= 1 && pool_factor(a) && pool_factor(d)) {
+        if (nc == 0 ? takes(a, d) : nc == 1 && unit_factor(a) && unit_factor(d)) {
             const cplx ratio = (a == 1.0) ? d : d / a;
             if (nc == 0) {
                 pool.g *= a;
