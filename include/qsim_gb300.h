@@ -109,7 +109,8 @@ typedef struct sim_plan_opts {
                                 n >= k + 7 (SIM_EINVAL otherwise).  Large registers (k = 6 from 26
                                 qubits, complex128 from 22): stretches of a unitary circuit that
                                 are predicted to be faster in register tiles run as tile passes. */
-    int32_t tile_qubits;     /* SIM_PLAN_STAGED: tile size log2 (0 = default) */
+    int32_t tile_qubits;     /* SIM_PLAN_STAGED: tile size log2 (0 = default: complex64 11 up to 18
+                                qubits, 12 up to 22, then 13; complex128 11 up to 19, then 12) */
     int32_t flags;           /* SIM_FLAG_* bits, 0 = defaults */
 } sim_plan_opts;
 
@@ -371,29 +372,31 @@ int sim_plan_features(int n, int dtype, const sim_gate *gates, size_t n_gates, i
 int sim_last_plan(sim_t s, int32_t *variants, size_t cap, size_t *len);
 
 /* ---- plan introspection (host only, no GPU needed) ---------------------------
- * sim_plan_describe: build the SIM_PLAN_STAGED schedule of a circuit for an
- *   n-qubit register of the given dtype without running it.  Outputs (any may
- *   be NULL): the number of tile passes, of ops (gate ops, layout changes,
- *   and phase ramps -- one per ramp, whatever its records), of register-layout
- *   changes, and the order in which the gates are applied (circuit indices;
+ * sim_plan_describe: what SIM_PLAN_STAGED makes of a circuit for an
+ *   n-qubit register of the given dtype, without running it.  Outputs (any may
+ *   be NULL): *passes, the tile passes that run (opts->tile_qubits 0 = the default
+ *   size, as in a run); and of the circuit's record schedule, the form the
+ *   cost model's features count, the number of ops (gate ops, layout changes,
+ *   and phase ramps -- one per ramp, whatever its records) and of register-layout
+ *   changes, and one valid order of the gates (circuit indices;
  *   a SWAP appears three times, lowered to three CNOT-type moves; identity
  *   gates are dropped) -- up to order_cap entries, the full length in
- *   *order_len.  SIM_EINVAL if no tile fits (n below 11) or a gate is invalid.
- *   With opts->plan = SIM_PLAN_FUSED (fuse_k 0 = 5): *passes gets the passes
+ *   *order_len.  (What a pass executes is its tile program,
+ *   sim_plan_tile_programs.)  SIM_EINVAL if no tile fits (n below 11) or a gate is invalid.
+ *   With opts->plan = SIM_PLAN_FUSED (fuse_k 0 = 5; complex128 4): *passes gets the passes
  *   the fused plan makes over the state (a multi-block pass counts once,
- *   see SIM_FLAG_MULTI_BLOCK_PASSES),
- *   *ops the fused blocks, if all of it runs in blocks; *layout_changes and
- *   *order_len are set to 0.
+ *   see SIM_FLAG_MULTI_BLOCK_PASSES; the tile passes of a large register count),
+ *   *ops the fused blocks; *layout_changes and *order_len are set to 0.
  *   Other plans: SIM_EUNSUPPORTED. */
 int sim_plan_describe(int n, int dtype, const sim_gate *gates, size_t n_gates, const sim_plan_opts *opts,
                       int64_t *passes, int64_t *ops, int64_t *layout_changes, int32_t *order, size_t order_cap,
                       size_t *order_len);
 
-/* sim_plan_staged_ops: the SIM_PLAN_STAGED schedule of a circuit, host only,
- *   for inspection and for checking the planner without a GPU (the record
- *   layout follows the library's version): which gates each pass applies, and
- *   one valid order and layout for them.  What the kernels run is compiled
- *   from the passes (sim_plan_tile_programs).  A tile is 2^M amplitudes: local
+/* sim_plan_staged_ops: the record schedule of a circuit in register tiles, host only:
+ *   one op per gate or phase ramp, the form the cost model's features count.  No
+ *   kernel runs it (sim_plan_tile_programs gives what they run); it is a valid
+ *   schedule of the same planner, for inspection and for checking that without a GPU (the record
+ *   layout follows the library's version).  A tile is 2^M amplitudes: local
  *   bits 0..4 are qubits 0..4, local bit 5 + i is the pass's high qubit i;
  *   256 threads hold 2^(M - 8) registers each.  Register layout l places
  *   register bit j and thread bit i on local bits given by the library's

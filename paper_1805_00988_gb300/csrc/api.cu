@@ -438,15 +438,22 @@ int sim_plan_describe(int n, int dtype, const sim_gate *gates, size_t n_gates, c
         if (layout_changes) *layout_changes = 0;
         if (order_len) *order_len = 0;
         int64_t blocks = 0, np = 0;
-        const int rc = describe_fused(n, gates, n_gates, opts->fuse_k ? opts->fuse_k : (dtype == SIM_C128 ? 4 : 5), &blocks, 0,
-                                      (opts->flags & SIM_FLAG_MULTI_BLOCK_PASSES) != 0, &np);
+        const int rc = describe_fused_run(n, dtype, gates, n_gates, opts->fuse_k ? opts->fuse_k : (dtype == SIM_C128 ? 4 : 5),
+                                          (opts->flags & SIM_FLAG_MULTI_BLOCK_PASSES) != 0, &blocks, &np);
         if (passes) *passes = np;
         if (ops) *ops = blocks;
         return rc;
     }
     if (plan != SIM_PLAN_STAGED) return fail(SIM_EUNSUPPORTED, "sim_plan_describe: staged or fused plans only");
-    return describe_staged(n, dtype, gates, n_gates, opts->tile_qubits, passes, ops, layout_changes, order,
-                           order_cap, order_len);
+    if (int rc = describe_staged(n, dtype, gates, n_gates, opts->tile_qubits, nullptr, ops, layout_changes, order,
+                                 order_cap, order_len))
+        return rc;
+    if (passes) {
+        std::vector<SGate> g;
+        lower_renamed(gates, n_gates, n, &g);
+        *passes = tile_passes(g, n, dtype, opts->tile_qubits);
+    }
+    return SIM_OK;
 }
 
 int sim_plan_staged_ops(int n, int dtype, const sim_gate *gates, size_t n_gates, int tile_qubits, sim_tile_op *ops,

@@ -1690,13 +1690,11 @@ int run_fused(qsim_state *s, const std::vector<SGate> &g, int depth, bool allow_
 
 }  // namespace
 
-int describe_fused(int n, const sim_gate *gates, size_t n_gates, int k, int64_t *blocks_out, int depth, bool multi,
-                   int64_t *passes_out)
+// blocks, and passes that apply them, of one run_fused call
+static void count_blocks(const std::vector<SGate> &g, int n, int k, int d, bool multi, int64_t *blocks_out,
+                         int64_t *passes_out)
 {
-    std::vector<SGate> g;
-    lower_gates(gates, n_gates, &g);
     // the same schedule as the run: the first group's blocks at depth <= 2
-    const int d = depth > 0 ? depth : kRunDepth;
     BlockPlanner planner(g, k, n, std::min(d, 2));
     int64_t nb = 0, np = 0;
     for (size_t grp = 0;; ++grp) {
@@ -1712,8 +1710,17 @@ int describe_fused(int n, const sim_gate *gates, size_t n_gates, int k, int64_t 
         nb += (int64_t)blocks.size();
         for (size_t i = 0; i < blocks.size(); ++i) np += second[i] ? 0 : 1;
     }
-    if (blocks_out) *blocks_out = nb;
-    if (passes_out) *passes_out = np;
+    *blocks_out += nb;
+    *passes_out += np;
+}
+
+int describe_fused(int n, const sim_gate *gates, size_t n_gates, int k, int64_t *blocks_out, int depth)
+{
+    std::vector<SGate> g;
+    lower_gates(gates, n_gates, &g);
+    int64_t passes = 0;
+    *blocks_out = 0;
+    count_blocks(g, n, k, depth, false, blocks_out, &passes);
     return SIM_OK;
 }
 
@@ -1818,24 +1825,63 @@ static std::vector<int> mixed_choice(const std::vector<SGate> &all, size_t ng, s
     return choice;
 }
 
-static int run_mixed(qsim_state *s, const std::vector<SGate> &all, int k)
+// run(tiles, gates) for each stretch of the mixed plan, in order, until one fails
+template <typename F>
+static int for_stretches(const std::vector<SGate> &all, int n, int dtype, int k, F run)
 {
-    if (s->dtype == SIM_C128 && s->n < 20) return run_tiles(s, all);
+    if (dtype == SIM_C128 && n < 20) return run(true, all);
     // the renaming's last exchanges of places run as tile passes
     size_t ng = all.size();
     while (ng && all[ng - 1].op == OP_SWAP) --ng;
-    const size_t W = (size_t)std::max(64, 8 * s->n), nw = (ng + W - 1) / W;
-    const std::vector<int> choice = mixed_choice(all, ng, W, s->n, s->dtype, k);
+    const size_t W = (size_t)std::max(64, 8 * n), nw = (ng + W - 1) / W;
+    const std::vector<int> choice = mixed_choice(all, ng, W, n, dtype, k);
     for (size_t w = 0; w < nw;) {
         size_t e = w + 1;
         while (e < nw && choice[e] == choice[w]) ++e;
         const size_t end = (e == nw && choice[w]) ? all.size() : std::min(ng, e * W);
         const std::vector<SGate> g(all.begin() + (long)(w * W), all.begin() + (long)end);
-        if (int rc = choice[w] ? run_tiles(s, g) : run_blocks(s, g, k)) return rc;
+        if (int rc = run(choice[w] != 0, g)) return rc;
         w = e;
     }
     if (ng < all.size() && (nw == 0 || !choice[nw - 1]))
-        return run_tiles(s, std::vector<SGate>(all.begin() + (long)ng, all.end()));
+        return run(true, std::vector<SGate>(all.begin() + (long)ng, all.end()));
+    return SIM_OK;
+}
+
+static int run_mixed(qsim_state *s, const std::vector<SGate> &all, int k)
+{
+    return for_stretches(all, s->n, s->dtype, k, [&](bool tiles, const std::vector<SGate> &g) {
+        return tiles ? run_tiles(s, g) : run_blocks(s, g, k);
+    });
+}
+
+// the gates of a circuit that runs mixed (false: it runs in blocks)
+static bool lower_mixed(const sim_gate *gates, size_t n_gates, int n, int dtype, int k, bool learned, std::vector<SGate> *g)
+{
+    if (!fused_mixes(n, dtype, k, learned)) return false;
+    lower_renamed(gates, n_gates, n, g);
+    // unitary circuits only: what the blocks' scales refuse stays refused
+    for (const SGate &x : *g)
+        if (x.op != OP_SWAP && !(std::abs(sgate_norm_bound(x) - 1.0) < 1e-6)) {
+            g->clear();
+            return false;
+        }
+    return true;
+}
+
+int describe_fused_run(int n, int dtype, const sim_gate *gates, size_t n_gates, int k, bool multi, int64_t *blocks_out,
+                       int64_t *passes_out)
+{
+    *blocks_out = *passes_out = 0;
+    std::vector<SGate> all;
+    if (!multi && lower_mixed(gates, n_gates, n, dtype, k, false, &all))
+        return for_stretches(all, n, dtype, k, [&](bool tiles, const std::vector<SGate> &g) {
+            if (tiles) *passes_out += tile_passes(g, n, dtype, 0);
+            else count_blocks(g, n, k, kRunDepth, false, blocks_out, passes_out);
+            return (int)SIM_OK;
+        });
+    lower_gates(gates, n_gates, &all);
+    count_blocks(all, n, k, kRunDepth, multi, blocks_out, passes_out);
     return SIM_OK;
 }
 
@@ -1863,15 +1909,7 @@ int apply_circuit_fused(qsim_state *s, const sim_gate *gates, size_t n_gates, co
     if (s->n < k + 7) return fail(SIM_EINVAL, "fused plan: needs n >= fuse_k + 7 (one CTA covers 128 rows)");
     std::vector<SGate> g;
     const bool multi = (o.flags & SIM_FLAG_MULTI_BLOCK_PASSES) != 0;
-    if (!multi && fused_mixes(s->n, s->dtype, k, o.plan == SIM_PLAN_LEARNED)) {
-        lower_renamed(gates, n_gates, s->n, &g);
-        // unitary circuits only: what the blocks' scales refuse stays refused
-        bool unitary = true;
-        for (size_t i = 0; i < g.size() && unitary; ++i)
-            unitary = g[i].op == OP_SWAP || std::abs(sgate_norm_bound(g[i]) - 1.0) < 1e-6;
-        if (unitary) return run_mixed(s, g, k);
-        g.clear();
-    }
+    if (!multi && lower_mixed(gates, n_gates, s->n, s->dtype, k, o.plan == SIM_PLAN_LEARNED, &g)) return run_mixed(s, g, k);
     lower_gates(gates, n_gates, &g);
     if (g.empty()) return SIM_OK;
     switch (k) {

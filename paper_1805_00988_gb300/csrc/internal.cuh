@@ -212,6 +212,8 @@ int apply_sgates_fused(qsim_state *s, const std::vector<SGate> &g, const double 
 // amplitudes (host only)
 int run_tiles(qsim_state *s, const std::vector<SGate> &g);
 double tile_cost(const std::vector<SGate> &g, int n, int dtype);
+// the tile passes such a run makes (tile_qubits 0: the default size)
+int64_t tile_passes(const std::vector<SGate> &g, int n, int dtype, int tile_qubits);
 // registers from this size on: the fused plan with the largest blocks takes
 // tile passes for the stretches they are predicted to be faster on
 bool fused_mixes(int n, int dtype, int k, bool learned);
@@ -221,13 +223,15 @@ int plan_features(int n, int dtype, const sim_gate *gates, size_t n_gates, int v
 // the learned plan's variant per window for a complex64 register with a cost
 // model (also stored as the handle's last plan)
 int learned_choose(qsim_state *s, const sim_gate *gates, size_t n_gates, std::vector<int> *best);
-// blocks of the fused plan (depth 0 = the depth the plan runs with) and, when
-// passes_out is given, the passes over the state (multi-block passes pair
-// blocks when multi is set)
-int describe_fused(int n, const sim_gate *gates, size_t n_gates, int k, int64_t *blocks_out, int depth = 0,
-                   bool multi = true, int64_t *passes_out = nullptr);
+// blocks of a circuit under the block planner of the given depth
+int describe_fused(int n, const sim_gate *gates, size_t n_gates, int k, int64_t *blocks_out, int depth);
+// what SIM_PLAN_FUSED runs: its blocks and its passes over the state (multi-block
+// passes pair blocks when multi is set; tile passes of the mixed form count)
+int describe_fused_run(int n, int dtype, const sim_gate *gates, size_t n_gates, int k, bool multi, int64_t *blocks_out,
+                       int64_t *passes_out);
 // the (cheaper) planner depth the learned plan's features are computed with
 int fused_feature_depth();
+// the record schedule (the cost model's features count its passes, ops and layout changes)
 int describe_staged(int n, int dtype, const sim_gate *gates, size_t n_gates, int tile_qubits, int64_t *passes,
                     int64_t *ops, int64_t *layout_changes, int32_t *order, size_t order_cap, size_t *order_len);
 int encode_staged(int n, int dtype, const sim_gate *gates, size_t n_gates, int tile_qubits, sim_tile_op *ops,

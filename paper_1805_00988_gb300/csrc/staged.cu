@@ -162,11 +162,27 @@ int run_tiles(qsim_state *s, const std::vector<SGate> &g)
     return s->dtype == SIM_C128 ? run_staged<double>(s, g, M) : run_staged<float>(s, g, M);
 }
 
+int64_t tile_passes(const std::vector<SGate> &g, int n, int dtype, int tile_qubits)
+{
+    const bool c128 = dtype == SIM_C128;
+    const int M = tile_qubits ? tile_qubits : default_tile(n, c128);
+    int64_t count = 0;
+    Program p;
+    if (c128) {
+        TilePlanner<double> plan(g, n, M, 1, false, false);
+        while (plan.next(&p)) ++count;
+    } else {
+        TilePlanner<float> plan(g, n, M, 2, false, false);
+        while (plan.next(&p)) ++count;
+    }
+    return count;
+}
+
 int describe_staged(int n, int dtype, const sim_gate *gates, size_t n_gates, int tile_qubits, int64_t *passes,
                     int64_t *ops, int64_t *layout_changes, int32_t *order, size_t order_cap, size_t *order_len)
 {
     const bool c128 = dtype == SIM_C128;
-    int M = tile_qubits ? tile_qubits : (c128 ? 11 : 13);
+    int M = tile_qubits ? tile_qubits : default_tile(n, c128);
     if (M > n || M < 11 || M > (c128 ? 12 : 13)) return fail(SIM_EINVAL, "describe: no staged tile fits");
     std::vector<SGate> g;
     lower_gates(gates, n_gates, &g);
@@ -186,7 +202,7 @@ int encode_staged(int n, int dtype, const sim_gate *gates, size_t n_gates, int t
                   size_t ops_cap, int32_t *info, size_t info_cap, size_t *n_ops, size_t *n_passes)
 {
     const bool c128 = dtype == SIM_C128;
-    int M = tile_qubits ? tile_qubits : (c128 ? 11 : 13);
+    int M = tile_qubits ? tile_qubits : default_tile(n, c128);
     if (M > n || M < 11 || M > (c128 ? 12 : 13)) return fail(SIM_EINVAL, "encode: no staged tile fits");
     std::vector<SGate> g;
     lower_gates(gates, n_gates, &g);
@@ -232,7 +248,7 @@ int export_tile_programs(int n, int dtype, const sim_gate *gates, size_t n_gates
                          size_t words_cap, int32_t *info, size_t info_cap, size_t *n_words, size_t *n_passes)
 {
     const bool c128 = dtype == SIM_C128;
-    int M = tile_qubits ? tile_qubits : (c128 ? 11 : 13);
+    int M = tile_qubits ? tile_qubits : default_tile(n, c128);
     if (M > n || M < 11 || M > (c128 ? 12 : 13)) return fail(SIM_EINVAL, "tile programs: no staged tile fits");
     std::vector<SGate> g;
     lower_renamed(gates, n_gates, n, &g);

@@ -254,7 +254,7 @@ _sig("sim_plan_staged_ops", [_i32, _i32, P, _sz, _i32, P, _sz, P, _sz, P, P])
 
 
 def sim_plan_staged_ops(n: int, dtype: int, sim_gates: np.ndarray, tile_qubits: int = 0):
-    """The staged plan's encoded op records and per-pass geometry (host only):
+    """The record schedule of a circuit in register tiles and its per-pass geometry (host only):
     returns (ops as SIM_TILE_OP_DTYPE records, info as an int32 array of
     shape (passes, SIM_TILE_PASS_INFO))."""
     g = np.ascontiguousarray(sim_gates, dtype=SIM_GATE_DTYPE)
@@ -288,7 +288,8 @@ def sim_plan_tile_programs(n: int, dtype: int, sim_gates: np.ndarray, tile_qubit
 
 
 def sim_plan_describe(n: int, dtype: int, sim_gates: np.ndarray, opts: sim_plan_opts):
-    """Host-only: (passes, ops, layout_changes, order) of the staged schedule."""
+    """Host-only: the passes of a staged or fused run; (ops, layout_changes,
+    order) of the staged record schedule, or the fused blocks as ops."""
     g = np.ascontiguousarray(sim_gates, dtype=SIM_GATE_DTYPE)
     passes, ops, lc = ctypes.c_int64(), ctypes.c_int64(), ctypes.c_int64()
     ln = ctypes.c_size_t()
