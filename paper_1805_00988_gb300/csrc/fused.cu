@@ -30,6 +30,7 @@
 // records SIM_ETIMEOUT in a device status word, frees its tensor memory and
 // returns.
 #include <algorithm>
+#include <complex>
 #include <cstring>
 #include <vector>
 
@@ -1383,6 +1384,17 @@ static double sgate_norm_bound(const SGate &g)
     return g.ctrl ? std::max(sig, 1.0) : sig;
 }
 
+// The 2 x 2 matrix (whatever the controls) is unitary to single precision: its columns
+// are orthogonal and of length 1, so both singular values are 1.  The norm bound
+// alone would let contractions and projectors pass.
+static bool sgate_unitary(const SGate &g)
+{
+    const std::complex<double> a(g.m[0], g.m[1]), b(g.m[2], g.m[3]), c(g.m[4], g.m[5]), d(g.m[6], g.m[7]);
+    constexpr double tol = 1e-6;
+    return std::abs(std::norm(a) + std::norm(c) - 1.0) < tol && std::abs(std::norm(b) + std::norm(d) - 1.0) < tol &&
+           std::abs(std::conj(a) * b + std::conj(c) * d) < tol;
+}
+
 // k = 6: the exponent we of the power-of-two scale of a block's W, and the
 // block's norm bound (every entry of U_blk = G_m ... G_1, and so of its real
 // form W, is at most the spectral norm of U_blk, which is at most the product
@@ -1862,7 +1874,7 @@ static bool lower_mixed(const sim_gate *gates, size_t n_gates, int n, int dtype,
     lower_renamed(gates, n_gates, n, g);
     // unitary circuits only: what the blocks' scales refuse stays refused
     for (const SGate &x : *g)
-        if (x.op != OP_SWAP && !(std::abs(sgate_norm_bound(x) - 1.0) < 1e-6)) {
+        if (x.op != OP_SWAP && !sgate_unitary(x)) {
             g->clear();
             return false;
         }
