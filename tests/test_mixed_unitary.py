@@ -1,9 +1,6 @@
 """Only unitary circuits take the mixed form of the fused plan (blocks and register
 tiles).  A plan described with multi-block passes asked for never mixes, so it gives the
-blocks that a circuit with a contraction must run as.
-
-GPU tolerances: those of the fused plans' tests, 1e-4 (complex64) and 1e-11 (complex128)
-of the largest amplitude."""
+blocks that a circuit with a contraction must run as, and on the GPU the same bits."""
 import numpy as np
 import pytest
 
@@ -54,18 +51,16 @@ def test_contractions_run_in_blocks(dt, n, k, kind):
         pytest.skip("no GPU")
     from paper_1805_00988_gb300 import costmodel, sim
     g = C.concat([circuit(kind, n), *extra("contraction", n) * 60, C.gate("x", 3)])
-    ref = sim.State(n, "c128")
-    sim.sim_set_basis_state(ref.h, 5)
-    ref.apply(g, plan="per_gate")
     st = sim.State(n, dt)
     model = costmodel.load()[0]
     sim.sim_set_cost_model(st.h, model)
+    sim.sim_set_basis_state(st.h, 5)
+    st.apply(g, plan="fused", fuse_k=k, flags=sim.SIM_FLAG_MULTI_BLOCK_PASSES)
+    blocks = st.tensor.clone()
     sim.sim_profile_enable(st.h, True)
     for plan, kw in (("fused", {"fuse_k": k}), ("learned", {})):
         sim.sim_set_basis_state(st.h, 5)
         st.apply(g, plan=plan, **kw)
         assert "staged" not in sim.sim_profile_read(st.h)
-        d = (st.tensor.to(torch.complex128) - ref.tensor).abs().max().item()
-        assert d <= (1e-11 if dt == "c128" else 1e-4) * ref.tensor.abs().max().item(), plan
+        assert torch.equal(st.tensor, blocks), plan
     st.close()
-    ref.close()
