@@ -12,9 +12,9 @@
 // is an inverse CDF over the FP64 prefix of |a_j|^2 that is never
 // materialised for the whole state: sums per sub-block of 256 amplitudes and
 // per block of 32 sub-blocks (one read of the state), one scan over the block
-// sums, shots bucketed by block (counting sort), then per shot one warp picks
-// the sub-block from the block's sub-sums and scans only those 256
-// amplitudes (2 KB of complex64 per shot instead of the whole block).
+// sums, then per shot a search of the block, of the sub-block, of its eighth
+// and of the amplitude (256 bytes of complex64 per shot, or 2 KB where the pass has not
+// written the sums of the eighths, instead of the whole block).
 #include <cmath>
 
 #include "f32x2.cuh"
@@ -1023,7 +1023,83 @@ __device__ __forceinline__ int lane_locate(const double2 x[4], int gl, double ta
 // the block (bexcl, bincl), the sub-block (cum, inclusive within the block), the
 // eighth of it, the amplitude.  Where rounding leaves no crossing (t within an ulp of a
 // boundary), the last one with non-zero probability is taken.
-//
+
+// the tables of the first two levels
+struct ShotTables {
+    uint32_t nsub;
+    uint64_t nb;
+    const double *bexcl, *bincl, *cum;
+    const uint64_t *last;
+};
+
+// the sub-block (counted over the register) that holds t; d = t relative to its start
+__device__ __forceinline__ uint64_t find_sub(const ShotTables &T, double t, double &d)
+{
+    uint64_t lo = 0, hi = T.nb;
+    while (lo < hi) {
+        const uint64_t mid = (lo + hi) >> 1;
+        if (above(T.bincl[mid], t)) hi = mid; else lo = mid + 1;
+    }
+    const uint64_t b = lo < T.nb ? lo : *T.last;
+    const double be = T.bexcl[b];
+    const double *P = T.cum + b * T.nsub;
+    uint32_t j = 0, je = T.nsub;
+    while (j < je) {
+        const uint32_t mid = (j + je) >> 1;
+        if (above(be + P[mid], t)) je = mid; else j = mid + 1;
+    }
+    if (j == T.nsub)
+        for (--j; j > 0 && !(P[j] > P[j - 1]);) --j;
+    d = t - (be + (j > 0 ? P[j - 1] : 0.0));
+    return b * T.nsub + j;
+}
+
+// the last eighth that is not empty and starts at or before the target; d becomes relative to it
+__device__ __forceinline__ uint32_t find_eighth(const double ev[8], double &d)
+{
+    double acc = 0.0, gp = 0.0;
+    int g = -1;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        if (above(ev[k], 0.0) && (g < 0 || !above(acc, d))) {
+            g = k;
+            gp = acc;
+        }
+        if (k < 7) acc += ev[k];
+    }
+    d -= gp;
+    return (uint32_t)max(g, 0);
+}
+
+// the amplitude within the eighth, from the crossing in each of its eight lanes (-1: none)
+template <typename V, int NV>
+__device__ __forceinline__ uint32_t find_amplitude(const V (&x)[NV], int hit, int gr)
+{
+    uint32_t fl = (__ballot_sync(0xffffffffu, hit >= 0) >> (8 * gr)) & 0xffu;
+    if (__any_sync(0xffffffffu, fl == 0)) {        // no crossing: the last one that is not zero
+        int nz = -1;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            if constexpr (NV == 2) {
+                const float4 &v = x[e >> 1];
+                if ((e & 1) ? (v.z != 0.f || v.w != 0.f) : (v.x != 0.f || v.y != 0.f)) nz = e;
+            } else {
+                double p2 = 0.0;
+                acc_sq<double>(p2, x[e].x, x[e].y);
+                if (p2 > 0.0) nz = e;
+            }
+        }
+        const uint32_t nl = (__ballot_sync(0xffffffffu, nz >= 0) >> (8 * gr)) & 0xffu;
+        if (fl == 0) {
+            hit = max(nz, 0);
+            fl = nl ? 1u << (31 - __clz(nl)) : 1u;
+        }
+    }
+    const int L = __ffs(fl) - 1;
+    return (uint32_t)(4 * L + __shfl_sync(0xffffffffu, hit, 8 * gr + L));
+}
+
+// Many shots: the pass over the state has left the sums of the eighths.
 // A lane looks up the first three levels of its own shot; then eight
 // lanes read the 32 amplitudes of a shot's eighth, four shots of the warp at a time.
 // The FP64 pipe (one warp instruction every 16 cycles per SM) is kept to what a lane
@@ -1034,12 +1110,9 @@ __device__ __forceinline__ int lane_locate(const double2 x[4], int gl, double ta
 // (0.55 the pass over the state) and 0.74.  The reads are as random as the shots
 // either way, 256 bytes (512) per shot.
 template <typename R>
-__global__ void __launch_bounds__(256) k_shots(const R *__restrict__ st, uint32_t nsub, uint64_t seed,
-                                               const double *__restrict__ bexcl, const double *__restrict__ bincl,
-                                               uint64_t nb, const double *__restrict__ total,
-                                               const uint64_t *__restrict__ last, const double *__restrict__ cum,
-                                               const double *__restrict__ eighth, uint64_t shots,
-                                               uint64_t *__restrict__ out)
+__global__ void __launch_bounds__(256) k_shots(const R *__restrict__ st, ShotTables T, uint64_t seed,
+                                               const double *__restrict__ total, const double *__restrict__ eighth,
+                                               uint64_t shots, uint64_t *__restrict__ out)
 {
     using V = typename std::conditional<sizeof(R) == 4, float4, double2>::type;
     constexpr int NV = sizeof(R) == 4 ? 2 : 4;         // 16-byte vectors of a lane's four amplitudes
@@ -1049,44 +1122,17 @@ __global__ void __launch_bounds__(256) k_shots(const R *__restrict__ st, uint32_
     const uint64_t step = (uint64_t)gridDim.x * blockDim.x;
     for (uint64_t c0 = (uint64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); c0 < shots; c0 += step) {
         const uint64_t s = min(c0 + (uint64_t)lane, shots - 1);
-        const double t = unif(seed, s) * tot;
-        uint64_t lo = 0, hi = nb;
-        while (lo < hi) {
-            const uint64_t mid = (lo + hi) >> 1;
-            if (above(bincl[mid], t)) hi = mid; else lo = mid + 1;
-        }
-        const uint64_t b = lo < nb ? lo : *last;
-        const double be = bexcl[b];
-        const double *P = cum + b * nsub;
-        uint32_t j = 0, je = nsub;
-        while (j < je) {
-            const uint32_t mid = (j + je) >> 1;
-            if (above(be + P[mid], t)) je = mid; else j = mid + 1;
-        }
-        if (j == nsub)
-            for (--j; j > 0 && !(P[j] > P[j - 1]);) --j;
-        const double d = t - (be + (j > 0 ? P[j - 1] : 0.0));
-        const uint64_t q = b * nsub + j;
-        // the last eighth that is not empty and starts at or before the target
+        double rel;
+        const uint64_t q = find_sub(T, unif(seed, s) * tot, rel);
         const double2 *e2 = reinterpret_cast<const double2 *>(eighth + 8 * q);
-        double ev[8], acc = 0.0, gp = 0.0;
+        double ev[8];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             const double2 y = e2[k];
             ev[2 * k] = y.x;
             ev[2 * k + 1] = y.y;
         }
-        int g = -1;
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            if (above(ev[k], 0.0) && (g < 0 || !above(acc, d))) {
-                g = k;
-                gp = acc;
-            }
-            if (k < 7) acc += ev[k];
-        }
-        const uint32_t part = (uint32_t)(q * 8) + (uint32_t)max(g, 0);   // 32 amplitudes each
-        const double rel = d - gp;
+        const uint32_t part = (uint32_t)(q * 8) + find_eighth(ev, rel);   // 32 amplitudes each
         Target tl = {0.f, 0.f, 0};
         if constexpr (sizeof(R) == 4) tl = split_target(rel);
         const V *av = reinterpret_cast<const V *>(st) + gl * NV;
@@ -1112,32 +1158,92 @@ __global__ void __launch_bounds__(256) k_shots(const R *__restrict__ st, uint32_
                                                 __shfl_sync(0xffffffffu, tl.e, i)});
             else
                 hit = lane_locate(x, gl, __shfl_sync(0xffffffffu, rel, i));
-            uint32_t fl = (__ballot_sync(0xffffffffu, hit >= 0) >> (8 * gr)) & 0xffu;
-            if (__any_sync(0xffffffffu, fl == 0)) {        // no crossing: the last one that is not zero
-                int nz = -1;
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    if constexpr (sizeof(R) == 4) {
-                        const float4 &v = x[e >> 1];
-                        if ((e & 1) ? (v.z != 0.f || v.w != 0.f) : (v.x != 0.f || v.y != 0.f)) nz = e;
-                    } else {
-                        double p2 = 0.0;
-                        acc_sq<double>(p2, x[e].x, x[e].y);
-                        if (p2 > 0.0) nz = e;
-                    }
-                }
-                const uint32_t nl = (__ballot_sync(0xffffffffu, nz >= 0) >> (8 * gr)) & 0xffu;
-                if (fl == 0) {
-                    hit = max(nz, 0);
-                    fl = nl ? 1u << (31 - __clz(nl)) : 1u;
-                }
-            }
-            const int L = __ffs(fl) - 1;
-            const uint32_t found = (uint32_t)(4 * L + __shfl_sync(0xffffffffu, hit, 8 * gr + L));
+            const uint32_t found = find_amplitude(x, hit, gr);
             const uint32_t mine = __shfl_sync(0xffffffffu, found, 8 * (lane & 3));
             if ((lane >> 2) == it) idx = mine;
         }
         if (c0 + (uint64_t)lane < shots) out[s] = (uint64_t)part * 32 + idx;
+    }
+}
+
+// sum of |a|^2 over the 32 amplitudes at p, by the operations of k_sub_sums
+__device__ __forceinline__ double eighth_sum(const float *p)
+{
+    const float4 *a4 = reinterpret_cast<const float4 *>(p);
+    double t = 0.0;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        float4 x[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) x[u] = a4[h * 8 + u];
+        float m = 0.f;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) m = absmax4(m, x[u]);
+        const Pow2 pw = pow2_for(m);
+        const pack2 sc = dup(pw.scale), nsc = dup(-pw.scale);
+#pragma unroll
+        for (int c = 0; c < 8; c += 4) {
+            Sq32 A;
+#pragma unroll
+            for (int u = c; u < c + 4; ++u) {
+                const Split2 q0 = square2(pk(x[u].x, x[u].y), sc, nsc);
+                const Split2 q1 = square2(pk(x[u].z, x[u].w), sc, nsc);
+                const float2 h0 = unpk(q0.nh), l0 = unpk(q0.l), h1 = unpk(q1.nh), l1 = unpk(q1.l);
+                A.add_split(h0.x, l0.x); A.add_split(h0.y, l0.y);
+                A.add_split(h1.x, l1.x); A.add_split(h1.y, l1.y);
+            }
+            t += widen_sum(A, pw.sh);
+        }
+    }
+    return t;
+}
+__device__ __forceinline__ double eighth_sum(const double *p)
+{
+    const double2 *a = reinterpret_cast<const double2 *>(p);
+    double t = 0.0;
+#pragma unroll
+    for (int e0 = 0; e0 < 32; e0 += 8) {
+        double2 x[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) x[u] = a[e0 + u];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) acc_sq<double>(t, x[u].x, x[u].y);
+    }
+    return t;
+}
+
+// Few shots for the register's size: the pass over the state has not written the eighths
+// (see kEighthsPer64), so eight lanes take one shot and form those of its sub-block
+// from all 256 amplitudes.
+template <typename R>
+__global__ void __launch_bounds__(256) k_shots_read(const R *__restrict__ st, ShotTables T, uint64_t seed,
+                                                    const double *__restrict__ total, uint64_t shots,
+                                                    uint64_t *__restrict__ out)
+{
+    using V = typename std::conditional<sizeof(R) == 4, float4, double2>::type;
+    constexpr int NV = sizeof(R) == 4 ? 2 : 4;
+    const double tot = *total;
+    if (!(tot > 0.0)) return;
+    const int lane = threadIdx.x & 31, gr = lane >> 3, gl = lane & 7;
+    const uint64_t step = (uint64_t)gridDim.x * (blockDim.x >> 3);
+    for (uint64_t c0 = ((uint64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31u)) >> 3; c0 < shots; c0 += step) {
+        const uint64_t s = min(c0 + (uint64_t)gr, shots - 1);
+        double rel, ev[8];
+        const uint64_t q = find_sub(T, unif(seed, s) * tot, rel);
+        __syncwarp();
+        const double e = eighth_sum(st + 2 * ((q << kSubLog) + 32 * (uint64_t)gl));
+#pragma unroll
+        for (int k = 0; k < 8; ++k) ev[k] = __shfl_sync(0xffffffffu, e, 8 * gr + k);
+        const uint64_t part = q * 8 + find_eighth(ev, rel);
+        const V *av = reinterpret_cast<const V *>(st) + part * (8 * NV) + gl * NV;
+        V x[NV];
+#pragma unroll
+        for (int u = 0; u < NV; ++u) x[u] = av[u];
+        int hit;
+        if constexpr (sizeof(R) == 4) hit = lane_locate(x, gl, split_target(rel));
+        else hit = lane_locate(x, gl, rel);
+        const uint32_t found = find_amplitude(x, hit, gr);
+        if (gl == 0 && c0 + (uint64_t)gr < shots) out[s] = part * 32 + found;
     }
 }
 
@@ -1318,6 +1424,16 @@ bool sample_observe_fused(const qsim_state *s)
     return s->dtype == SIM_C64 && s->n >= kSampleLog && SubGeo(1ull << kSampleLog).sub == 256;
 }
 
+// The pass over the state writes the sums of its eighths (8 bytes per 32 amplitudes:
+// 8-11 % of its time for complex64) where the shots pay for them: a shot reads 256 bytes
+// with them and 2 KB without (512 and 4 KB).  For a million shots, with / without (and
+// one shot in a warp, sorted by block, before there were eighths): complex64 28 qubits 0.80 / 1.26 (1.83)
+// ms, 30 2.31 / 2.65 (3.37), 33 16.2 / 15.2 (16.1); complex128 30 4.36 / 5.23 (7.84).  For 10^4:
+// 0.69 / 0.62 (0.65), 2.20 / 1.97 (2.01), 16.1 / 14.4 (14.6); 4.14 / 3.93 (3.96).  The two
+// are even at about one shot in 2300 amplitudes (complex64, 27 qubits and more) and
+// one in 3600-6700 (complex128).
+constexpr uint64_t kEighthsPer64 = 2048, kEighthsPer128 = 4096;
+
 int run_sample(qsim_state *s, uint64_t shots, uint64_t seed, uint64_t *out, int out_on_device, double *norm_out,
                double *expz_out)
 {
@@ -1335,15 +1451,22 @@ int run_sample(qsim_state *s, uint64_t shots, uint64_t seed, uint64_t *out, int 
     const bool full = sg.sub == (1u << kSubLog);
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t o = off; off += (bytes + 255) & ~(size_t)255; return o; };
-    const size_t o_cum = take(nb * sg.nsub * 8), o_eig = full ? take(nb * sg.nsub * 64) : 0;
+    const size_t o_cum = take(nb * sg.nsub * 8);
     const size_t o_bsum = take(nb * 8), o_bexcl = take(nb * 8), o_bincl = take(nb * 8), o_tot = take(4 * 8);
     const uint64_t nchunk = (nb + kScanChunk - 1) / kScanChunk;
     const size_t o_cs = take(2 * nchunk * 8);
     const size_t o_zpart = obs ? take(2 * nb * 8) : 0;
     const size_t o_out = out_on_device ? 0 : take(shots * 8);
+    const bool c128 = s->dtype == SIM_C128;
+    bool stored = full && shots >= N / (c128 ? kEighthsPer128 : kEighthsPer64);
+    const size_t o_eig = off;
     char *scratch = nullptr;
-    QSIM_CUDA(cudaMallocAsync((void **)&scratch, off, s->stream));
-    double *cum = (double *)(scratch + o_cum), *eighth = full ? (double *)(scratch + o_eig) : nullptr;
+    if (stored && cudaMallocAsync((void **)&scratch, off + nb * sg.nsub * 64, s->stream) != cudaSuccess) {
+        cudaGetLastError();
+        stored = false;                // the eighths do not fit beside the state: do without
+    }
+    if (!stored) QSIM_CUDA(cudaMallocAsync((void **)&scratch, off, s->stream));
+    double *cum = (double *)(scratch + o_cum), *eighth = stored ? (double *)(scratch + o_eig) : nullptr;
     double *bsum = (double *)(scratch + o_bsum), *bexcl = (double *)(scratch + o_bexcl);
     double *bincl = (double *)(scratch + o_bincl);
     double *tot = (double *)(scratch + o_tot), *zout = tot + 2;        // zout: two values
@@ -1351,8 +1474,8 @@ int run_sample(qsim_state *s, uint64_t shots, uint64_t seed, uint64_t *out, int 
     uint64_t *dout = out_on_device ? out : (uint64_t *)(scratch + o_out);
     double *cs = (double *)(scratch + o_cs);
     double *zpart = obs ? (double *)(scratch + o_zpart) : nullptr;
+    const ShotTables tables{sg.nsub, nb, bexcl, bincl, cum, last};
     int rc = SIM_OK;
-    const bool c128 = s->dtype == SIM_C128;
     do {
         launch_begin(s, KC_SAMPLE, (double)s->bytes);
         if (c128) k_sub_sums<double><<<(unsigned)nb, 256, 0, s->stream>>>((const double *)s->amps, bs, cum, bsum, eighth);
@@ -1370,15 +1493,17 @@ int run_sample(qsim_state *s, uint64_t shots, uint64_t seed, uint64_t *out, int 
         launch_begin(s, KC_SAMPLE);
         k_last_nonzero<<<1, 1024, 0, s->stream>>>(bsum, nb, last);
         if ((rc = launch_end(s, "last nonzero"))) break;
-        // per shot 32 amplitudes; a zero norm writes none
-        launch_begin(s, KC_SAMPLE, (double)shots * (full ? 32.0 : 0.0) * (c128 ? 16.0 : 8.0));
-        const unsigned grid = grid_for(shots, 256, s->num_sms);
-        if (full && c128)
-            k_shots<double><<<grid, 256, 0, s->stream>>>((const double *)s->amps, sg.nsub, seed, bexcl, bincl, nb, tot,
-                                                         last, cum, eighth, shots, dout);
+        // per shot 32 amplitudes (256 without the eighths); a zero norm writes none
+        launch_begin(s, KC_SAMPLE, (double)shots * (stored ? 32.0 : full ? 256.0 : 0.0) * (c128 ? 16.0 : 8.0));
+        const unsigned grid = grid_for(full && !stored ? 8 * shots : shots, 256, s->num_sms);
+        if (stored && c128)
+            k_shots<double><<<grid, 256, 0, s->stream>>>((const double *)s->amps, tables, seed, tot, eighth, shots, dout);
+        else if (stored)
+            k_shots<float><<<grid, 256, 0, s->stream>>>((const float *)s->amps, tables, seed, tot, eighth, shots, dout);
+        else if (full && c128)
+            k_shots_read<double><<<grid, 256, 0, s->stream>>>((const double *)s->amps, tables, seed, tot, shots, dout);
         else if (full)
-            k_shots<float><<<grid, 256, 0, s->stream>>>((const float *)s->amps, sg.nsub, seed, bexcl, bincl, nb, tot,
-                                                        last, cum, eighth, shots, dout);
+            k_shots_read<float><<<grid, 256, 0, s->stream>>>((const float *)s->amps, tables, seed, tot, shots, dout);
         else if (c128)
             k_shots_small<double><<<grid, 256, 0, s->stream>>>((const double *)s->amps, (uint32_t)N, seed, tot, shots,
                                                                dout);
