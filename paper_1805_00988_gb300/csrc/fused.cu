@@ -1758,6 +1758,10 @@ bool fused_mixes(int n, int dtype, int k, bool learned)
     return dtype == SIM_C128 ? k == 4 && (learned || n >= 22) : k == 6 && n >= 26;
 }
 
+// rotations and controlled exchanges, a third of the gates each or more: few gates
+// commute into a tile pass, and every exchange costs one as much as three rotations
+static bool ladder_like(size_t rot, size_t xch, size_t count) { return 3 * rot >= count && 3 * xch >= count; }
+
 static int run_blocks(qsim_state *s, const std::vector<SGate> &g, int k)
 {
     return k == 4 ? run_fused<4>(s, g, kRunDepth, false) : run_fused<6>(s, g, kRunDepth, false);
@@ -1785,13 +1789,15 @@ static std::vector<int> mixed_choice(const std::vector<SGate> &all, size_t ng, s
     std::vector<char> exact(nw, 0);
     const bool c128 = dtype == SIM_C128;
     for (size_t w = 0; w < nw; ++w) {
-        double rot = 0, xch = 0, cz = 0, cp = 0;
-        const size_t end = std::min(ng, (w + 1) * W);
+        double rot = 0, xch = 0, dense = 0, cz = 0, cp = 0;     // dense: exchanges that are not moves
+        const size_t end = std::min(ng, (w + 1) * W), count = end - w * W;
         for (size_t i = w * W; i < end; ++i) {
             const SGate &g = all[i];
             if (g.xq() && !g.ctrl) rot += g.op == OP_XPERM ? 0 : 1;
-            else if (g.xq()) xch += 1;
-            else if (g.ctrl) (g.m[6] == -1.0 && g.m[7] == 0.0 ? cz : cp) += 1;
+            else if (g.xq()) {
+                xch += 1;
+                dense += g.op != OP_XPERM;
+            } else if (g.ctrl) (g.m[6] == -1.0 && g.m[7] == 0.0 ? cz : cp) += 1;
         }
         if (c128) {
             tile[w] = 320 + 330 * rot + 80 * xch + 45 * cp + cz;
@@ -1800,20 +1806,29 @@ static std::vector<int> mixed_choice(const std::vector<SGate> &all, size_t ng, s
             tile[w] = 130 + 18.2 * rot + 38 * xch + 4 * cp + 0.5 * cz;
             block[w] = std::max({block_us, (n < 28 ? 22.5 : 17.2) * rot, block_us * (cz + cp) / 9.0});
         }
-        // (complex128 below 22 qubits: 0.2 ms of costing on a circuit of 2 ms)
-        exact[w] = 10 * xch > (double)(end - w * W) && !(c128 && n < 22);
+        // Costing takes 0.1 ms (22-qubit complex128 ladder: 1.23 ms without, 1.33 with it), so
+        // not below 22 qubits complex128, nor where the answer is certain: rotations and exchanges in equal
+        // parts (26 qubits, U3 + CNOT ladder: blocks 2.39 ms, tiles 3.98), or complex128
+        // tiles whose FP64 work alone is more than a block for every 2.5 gates.
+        const bool sure = c128 ? n < 22 || 320 + 330 * rot + 80 * (xch - dense) + 800 * dense > block_us * (double)count / 2.5
+                               : ladder_like((size_t)rot, (size_t)xch, count);
+        exact[w] = 10 * xch > (double)count && !sure;
     }
-    parallel_for(2 * nw, [&](size_t i) {
-        if (!exact[i / 2]) return;
-        const std::vector<SGate> g = window(i / 2);
+    // (waking the host threads takes 40 us: not for windows that a count answers)
+    std::vector<size_t> costed;
+    for (size_t w = 0; w < nw; ++w)
+        if (exact[w]) costed.push_back(w);
+    parallel_for(2 * costed.size(), [&](size_t i) {
+        const size_t w = costed[i / 2];
+        const std::vector<SGate> g = window(w);
         if (i & 1) {
-            tile[i / 2] = tile_cost(g, n, dtype);
+            tile[w] = tile_cost(g, n, dtype);
         } else {
             BlockPlanner planner(g, k, n, kFeatureDepth);
             Block b;
             int nb = 0;
             while (planner.next(&b)) ++nb;
-            block[i / 2] = block_us * nb;
+            block[w] = block_us * nb;
         }
     });
     // the cheapest sequence of choices (0: blocks, 1: tiles)
