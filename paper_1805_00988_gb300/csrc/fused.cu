@@ -30,7 +30,6 @@
 // records SIM_ETIMEOUT in a device status word, frees its tensor memory and
 // returns.
 #include <algorithm>
-#include <complex>
 #include <cstring>
 #include <vector>
 
@@ -1384,17 +1383,6 @@ static double sgate_norm_bound(const SGate &g)
     return g.ctrl ? std::max(sig, 1.0) : sig;
 }
 
-// The 2 x 2 matrix (whatever the controls) is unitary to single precision: its columns
-// are orthogonal and of length 1, so both singular values are 1.  The norm bound
-// alone would let contractions and projectors pass.
-static bool sgate_unitary(const SGate &g)
-{
-    const std::complex<double> a(g.m[0], g.m[1]), b(g.m[2], g.m[3]), c(g.m[4], g.m[5]), d(g.m[6], g.m[7]);
-    constexpr double tol = 1e-6;
-    return std::abs(std::norm(a) + std::norm(c) - 1.0) < tol && std::abs(std::norm(b) + std::norm(d) - 1.0) < tol &&
-           std::abs(std::conj(a) * b + std::conj(c) * d) < tol;
-}
-
 // k = 6: the exponent we of the power-of-two scale of a block's W, and the
 // block's norm bound (every entry of U_blk = G_m ... G_1, and so of its real
 // form W, is at most the spectral norm of U_blk, which is at most the product
@@ -1758,9 +1746,7 @@ bool fused_mixes(int n, int dtype, int k, bool learned)
     return dtype == SIM_C128 ? k == 4 && (learned || n >= 22) : k == 6 && n >= 26;
 }
 
-// rotations and controlled exchanges, a third of the gates each or more: few gates
-// commute into a tile pass, and every exchange costs one as much as three rotations
-static bool ladder_like(size_t rot, size_t xch, size_t count) { return 3 * rot >= count && 3 * xch >= count; }
+constexpr size_t kFewGates = 16;      // of a call or window: costed in no time
 
 static int run_blocks(qsim_state *s, const std::vector<SGate> &g, int k)
 {
@@ -1791,34 +1777,62 @@ static std::vector<int> mixed_choice(const std::vector<SGate> &all, size_t ng, s
     for (size_t w = 0; w < nw; ++w) {
         double rot = 0, xch = 0, dense = 0, cz = 0, cp = 0;     // dense: exchanges that are not moves
         const size_t end = std::min(ng, (w + 1) * W), count = end - w * W;
+        std::vector<uint64_t> pairs;           // qubits of the controlled phases
+        int deg[64] = {};
         for (size_t i = w * W; i < end; ++i) {
             const SGate &g = all[i];
             if (g.xq() && !g.ctrl) rot += g.op == OP_XPERM ? 0 : 1;
             else if (g.xq()) {
                 xch += 1;
                 dense += g.op != OP_XPERM;
-            } else if (g.ctrl) (g.m[6] == -1.0 && g.m[7] == 0.0 ? cz : cp) += 1;
+            } else if (g.ctrl) {
+                const bool sign = g.m[6] == -1.0 && g.m[7] == 0.0;
+                (sign ? cz : cp) += 1;
+                if (!sign) pairs.push_back(g.ctrl | (1ull << g.target));
+            }
         }
         if (c128) {
-            tile[w] = 320 + 330 * rot + 80 * xch + 45 * cp + cz;
+            // A ramp is bound by the FP64 pipe from 24 qubits on (below only a few pairs cost more
+            // than a block), and one applies the pairs of one
+            // qubit: as many as a greedy cover of the pairs takes (few in a QFT's window, nearly one
+            // each for scattered pairs: 27 qubits, 80 random diagonal gates 19.4 ms in
+            // tiles, 15.4 in blocks)
+            double ramps = 0;
+            if (n >= 24 || cp <= 4) {
+                for (uint64_t p : pairs)
+                    for (uint64_t m = p; m; m &= m - 1) ++deg[__builtin_ctzll(m)];
+                uint64_t cover = 0;
+                for (uint64_t p : pairs) {
+                    if (p & cover) continue;
+                    int best = __builtin_ctzll(p);
+                    for (uint64_t m = p; m; m &= m - 1)
+                        if (deg[__builtin_ctzll(m)] > deg[best]) best = __builtin_ctzll(m);
+                    cover |= 1ull << best;
+                }
+                ramps = __builtin_popcountll(cover);
+            }
+            tile[w] = 320 + 330 * rot + 80 * xch + std::max(45 * cp, 400 * ramps) + cz;
             block[w] = std::max({block_us, block_us * (rot + (n < 22 ? xch : 0)) / 6.0, block_us * (cz + cp) / 4.5});
         } else {
-            tile[w] = 130 + 18.2 * rot + 38 * xch + 4 * cp + 0.5 * cz;
+            tile[w] = 130 + 18.2 * rot + 38 * (xch - dense) + 70 * dense + 4 * cp + 0.5 * cz;
             block[w] = std::max({block_us, (n < 28 ? 22.5 : 17.2) * rot, block_us * (cz + cp) / 9.0});
         }
         // Costing takes 0.1 ms (22-qubit complex128 ladder: 1.23 ms without, 1.33 with it), so
         // not below 22 qubits complex128, nor where the answer is certain: rotations and exchanges in equal
         // parts (26 qubits, U3 + CNOT ladder: blocks 2.39 ms, tiles 3.98), or complex128
         // tiles whose FP64 work alone is more than a block for every 2.5 gates.
-        const bool sure = c128 ? n < 22 || 320 + 330 * rot + 80 * (xch - dense) + 800 * dense > block_us * (double)count / 2.5
-                               : ladder_like((size_t)rot, (size_t)xch, count);
+        bool sure = c128 && n < 22;
+        if (count >= kFewGates) {
+            if (!c128) sure = ladder_like((size_t)rot, (size_t)xch, count);
+            else if (320 + 330 * rot + 80 * (xch - dense) + 800 * dense > block_us * (double)count / 2.5) sure = true;
+        }
         exact[w] = 10 * xch > (double)count && !sure;
     }
     // (waking the host threads takes 40 us: not for windows that a count answers)
     std::vector<size_t> costed;
     for (size_t w = 0; w < nw; ++w)
         if (exact[w]) costed.push_back(w);
-    parallel_for(2 * costed.size(), [&](size_t i) {
+    auto cost = [&](size_t i) {
         const size_t w = costed[i / 2];
         const std::vector<SGate> g = window(w);
         if (i & 1) {
@@ -1830,7 +1844,12 @@ static std::vector<int> mixed_choice(const std::vector<SGate> &all, size_t ng, s
             while (planner.next(&b)) ++nb;
             block[w] = block_us * nb;
         }
-    });
+    };
+    if (ng < kFewGates) {
+        for (size_t i = 0; i < 2 * costed.size(); ++i) cost(i);
+    } else {
+        parallel_for(2 * costed.size(), cost);
+    }
     // the cheapest sequence of choices (0: blocks, 1: tiles)
     std::vector<std::array<double, 2>> best(nw);
     std::vector<std::array<int, 2>> from(nw);
@@ -1838,7 +1857,8 @@ static std::vector<int> mixed_choice(const std::vector<SGate> &all, size_t ng, s
         for (int c = 0; c < 2; ++c) {
             const double own = c ? tile[w] : block[w];
             if (w == 0) {
-                best[w][c] = own;
+                // complex64 blocks read the state's norm first (one H, 28 qubits: 1.15 ms in tiles, 1.50 in a block)
+                best[w][c] = own + (c == 0 && !c128 ? 80.0 : 0.0);
                 from[w][c] = c;
                 continue;
             }
@@ -1852,16 +1872,26 @@ static std::vector<int> mixed_choice(const std::vector<SGate> &all, size_t ng, s
     return choice;
 }
 
+// complex128 below 20 qubits: tiles, unless controlled dense gates are more than a third of
+// the gates (60 U3 gates, 37 of them controlled, 14 / 19 qubits: 367 / 638 us in tiles, 265 / 331 in blocks)
+static bool dense_exchanges(const std::vector<SGate> &g)
+{
+    size_t dense = 0;
+    for (const SGate &x : g) dense += x.ctrl && x.xq() && x.op != OP_XPERM;
+    return 3 * dense > g.size();
+}
+
 // run(tiles, gates) for each stretch of the mixed plan, in order, until one fails
 template <typename F>
 static int for_stretches(const std::vector<SGate> &all, int n, int dtype, int k, F run)
 {
-    if (dtype == SIM_C128 && n < 20) return run(true, all);
+    const bool small = dtype == SIM_C128 && n < 20;
+    if (small && !dense_exchanges(all)) return run(true, all);
     // the renaming's last exchanges of places run as tile passes
     size_t ng = all.size();
     while (ng && all[ng - 1].op == OP_SWAP) --ng;
-    const size_t W = (size_t)std::max(64, 8 * n), nw = (ng + W - 1) / W;
-    const std::vector<int> choice = mixed_choice(all, ng, W, n, dtype, k);
+    const size_t W = small ? std::max<size_t>(ng, 1) : (size_t)std::max(64, 8 * n), nw = (ng + W - 1) / W;
+    const std::vector<int> choice = small ? std::vector<int>(nw, 0) : mixed_choice(all, ng, W, n, dtype, k);
     for (size_t w = 0; w < nw;) {
         size_t e = w + 1;
         while (e < nw && choice[e] == choice[w]) ++e;
@@ -1889,7 +1919,7 @@ static bool lower_mixed(const sim_gate *gates, size_t n_gates, int n, int dtype,
     lower_renamed(gates, n_gates, n, g);
     // unitary circuits only: what the blocks' scales refuse stays refused
     for (const SGate &x : *g)
-        if (x.op != OP_SWAP && !sgate_unitary(x)) {
+        if (x.op != OP_SWAP && !unitary_2x2(x.m)) {
             g->clear();
             return false;
         }

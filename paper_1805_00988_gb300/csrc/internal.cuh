@@ -218,6 +218,10 @@ int64_t tile_passes(const std::vector<SGate> &g, int n, int dtype, int tile_qubi
 // tile passes for the stretches they are predicted to be faster on
 bool fused_mixes(int n, int dtype, int k, bool learned);
 bool learned_tiles_only(int n, int dtype);
+bool unitary_2x2(const double m[8]);               // to single precision
+// rotations and controlled exchanges, a third of the gates each or more: few gates
+// commute into a tile pass, and every exchange costs one as much as three rotations
+inline bool ladder_like(size_t rot, size_t xch, size_t count) { return 3 * rot >= count && 3 * xch >= count; }
 int apply_circuit_learned(qsim_state *s, const sim_gate *gates, size_t n_gates, const sim_plan_opts &o);
 int plan_features(int n, int dtype, const sim_gate *gates, size_t n_gates, int v, float *out);
 // the learned plan's variant per window for a complex64 register with a cost

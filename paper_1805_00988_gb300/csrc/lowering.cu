@@ -1,6 +1,7 @@
 // lowering.cu -- circuit gates to the planners' gate form.
 #include <algorithm>
 #include <cmath>
+#include <complex>
 #include <cstring>
 #include <vector>
 
@@ -12,6 +13,16 @@ bool commute(const SGate &a, const SGate &b)
 {
     const uint64_t shared = (a.xq() | a.dq()) & (b.xq() | b.dq());
     return (shared & (a.xq() | b.xq())) == 0;
+}
+
+// Columns orthogonal and of length 1, so both singular values are 1.  (The norm bound
+// alone would let contractions and projectors pass.)
+bool unitary_2x2(const double m[8])
+{
+    const std::complex<double> a(m[0], m[1]), b(m[2], m[3]), c(m[4], m[5]), d(m[6], m[7]);
+    constexpr double tol = 1e-6;
+    return std::abs(std::norm(a) + std::norm(c) - 1.0) < tol && std::abs(std::norm(b) + std::norm(d) - 1.0) < tol &&
+           std::abs(std::conj(a) * b + std::conj(c) * d) < tol;
 }
 
 // SWAP(a, b) with controls c = CNOT(b -> a) . X(target b; controls c + a) . CNOT(b -> a)

@@ -1944,7 +1944,7 @@ double pass_cost(const TilePass &tp)
         case IR_PERM: t += D ? 80.0 : 37.0; break;
         case IR_RAMP: t += D ? 400.0 : 23.0; break;
         case IR_CSHEARS: t += D ? 430.0 : 12.0; break;
-        case IR_XCH: t += D && ((o.arg >> 3) & 3u) == SK_DENSE ? 800.0 : 18.0; break;
+        case IR_XCH: t += ((o.arg >> 3) & 3u) == SK_XPERM ? 18.0 : ((o.arg >> 3) & 3u) == SK_DENSE && D ? 800.0 : 50.0; break;
         default: t += D ? 400.0 : 18.0; break;
         }
     }
