@@ -268,6 +268,7 @@ int apply_circuit_learned(qsim_state *s, const sim_gate *gates, size_t n_gates, 
         const size_t first = win[w].first, count = win[e - 1].first + win[e - 1].count - first;
         sim_plan_opts vo;
         variant_opts(best[w] < 0 ? 0 : best[w], &vo);
+        if (vo.plan == SIM_PLAN_STAGED) vo.tile_qubits = 0;   // the size the gates ask for
         int rc;
         if (vo.plan == SIM_PLAN_PER_GATE) {
             rc = SIM_OK;

@@ -147,25 +147,34 @@ double tile_cost(const std::vector<SGate> &g, int n, int dtype)
 // The tile size when the caller leaves it open.  Small tiles give small
 // registers more CTAs and shorter programs: 14 qubits, depth-20 random circuit
 // 274 / 307 / 338 us with 11- / 12- / 13-qubit tiles, 18 qubits 385 / 418 / 456, 20
-// qubits 440 / 458 / 500; 22 qubits 839 / 798 / 858; from 23 on 13 qubits win
-// on most circuits (fewer passes).  complex128: 12 qubits wherever they fit
-// (26-qubit QFT 24.3 against 25.3 ms).
-static int default_tile(int n, bool c128)
+// qubits 440 / 458 / 500; 22 qubits 839 / 798 / 858.  23 to 25 qubits: 12 and 13 are within
+// 6 % on Haar layers, QFTs, ladders and reversible circuits, and 12 takes a fifth to a
+// quarter less on phases and random gates (24 qubits: 223 / 300 and 814 / 1128 us).  Above, 13
+// saves passes that HBM bounds (28 qubits, Haar layers 13.1 / 12.4 ms, reversible 6.8 / 6.0), except
+// where controlled gates other than moves are more than an eighth: each costs every
+// amplitude a masked multiply, dearer with 64 amplitudes a thread (random gates, 27
+// qubits 7.1 / 9.4 ms, 28 14.0 / 18.2; they took 8.2 and 16.5 before tile programs).
+// complex128: 12 qubits wherever they fit (26-qubit QFT 24.3 against 25.3 ms).
+static int open_tile(const std::vector<SGate> &g, int n, bool c128)
 {
     if (c128) return n >= 20 ? 12 : 11;
-    return n <= 18 ? 11 : n <= 22 ? 12 : 13;
+    if (n <= 25) return n <= 18 ? 11 : 12;
+    size_t masked = 0;
+    for (const SGate &x : g)
+        masked += x.xq() ? x.ctrl && x.op != OP_XPERM && x.op != OP_SWAP : __builtin_popcountll(x.ctrl) >= 2;
+    return 8 * masked > g.size() ? 12 : 13;
 }
 
 int run_tiles(qsim_state *s, const std::vector<SGate> &g)
 {
-    const int M = default_tile(s->n, s->dtype == SIM_C128);
+    const int M = open_tile(g, s->n, s->dtype == SIM_C128);
     return s->dtype == SIM_C128 ? run_staged<double>(s, g, M) : run_staged<float>(s, g, M);
 }
 
 int64_t tile_passes(const std::vector<SGate> &g, int n, int dtype, int tile_qubits)
 {
     const bool c128 = dtype == SIM_C128;
-    const int M = tile_qubits ? tile_qubits : default_tile(n, c128);
+    const int M = tile_qubits ? tile_qubits : open_tile(g, n, c128);
     int64_t count = 0;
     Program p;
     if (c128) {
@@ -182,9 +191,14 @@ int describe_staged(int n, int dtype, const sim_gate *gates, size_t n_gates, int
                     int64_t *ops, int64_t *layout_changes, int32_t *order, size_t order_cap, size_t *order_len)
 {
     const bool c128 = dtype == SIM_C128;
-    int M = tile_qubits ? tile_qubits : default_tile(n, c128);
-    if (M > n || M < 11 || M > (c128 ? 12 : 13)) return fail(SIM_EINVAL, "describe: no staged tile fits");
     std::vector<SGate> g;
+    int M = tile_qubits;
+    if (!M) {
+        lower_renamed(gates, n_gates, n, &g);     // as a run has them
+        M = open_tile(g, n, c128);
+        g.clear();
+    }
+    if (M > n || M < 11 || M > (c128 ? 12 : 13)) return fail(SIM_EINVAL, "describe: no staged tile fits");
     lower_gates(gates, n_gates, &g);
     std::vector<Pass> ps = form_passes(g, n, M);
     PlanBuilder<double> pb{n, M, M - kThrBits, c128 ? 1 : 2, {}, {}, 0};
@@ -202,9 +216,14 @@ int encode_staged(int n, int dtype, const sim_gate *gates, size_t n_gates, int t
                   size_t ops_cap, int32_t *info, size_t info_cap, size_t *n_ops, size_t *n_passes)
 {
     const bool c128 = dtype == SIM_C128;
-    int M = tile_qubits ? tile_qubits : default_tile(n, c128);
-    if (M > n || M < 11 || M > (c128 ? 12 : 13)) return fail(SIM_EINVAL, "encode: no staged tile fits");
     std::vector<SGate> g;
+    int M = tile_qubits;
+    if (!M) {
+        lower_renamed(gates, n_gates, n, &g);     // as a run has them
+        M = open_tile(g, n, c128);
+        g.clear();
+    }
+    if (M > n || M < 11 || M > (c128 ? 12 : 13)) return fail(SIM_EINVAL, "encode: no staged tile fits");
     lower_gates(gates, n_gates, &g);
     std::vector<Pass> ps = form_passes(g, n, M);
     PlanBuilder<double> pb{n, M, M - kThrBits, c128 ? 1 : 2, {}, {}, 0};
@@ -248,10 +267,10 @@ int export_tile_programs(int n, int dtype, const sim_gate *gates, size_t n_gates
                          size_t words_cap, int32_t *info, size_t info_cap, size_t *n_words, size_t *n_passes)
 {
     const bool c128 = dtype == SIM_C128;
-    int M = tile_qubits ? tile_qubits : default_tile(n, c128);
-    if (M > n || M < 11 || M > (c128 ? 12 : 13)) return fail(SIM_EINVAL, "tile programs: no staged tile fits");
     std::vector<SGate> g;
     lower_renamed(gates, n_gates, n, &g);
+    int M = tile_qubits ? tile_qubits : open_tile(g, n, c128);
+    if (M > n || M < 11 || M > (c128 ? 12 : 13)) return fail(SIM_EINVAL, "tile programs: no staged tile fits");
     const std::vector<Program> ps = compile_passes<double>(g, n, M, c128 ? 1 : 2);
     size_t at = 0;
     for (size_t p = 0; p < ps.size(); ++p) {
@@ -277,7 +296,9 @@ int export_tile_programs(int n, int dtype, const sim_gate *gates, size_t n_gates
 int apply_circuit_staged(qsim_state *s, const sim_gate *gates, size_t n_gates, const sim_plan_opts &o)
 {
     const bool c128 = s->dtype == SIM_C128;
-    int M = o.tile_qubits ? o.tile_qubits : default_tile(s->n, c128);
+    std::vector<SGate> g;
+    lower_renamed(gates, n_gates, s->n, &g);
+    int M = o.tile_qubits ? o.tile_qubits : open_tile(g, s->n, c128);
     if (M > s->n) M = (s->n >= 11) ? 11 : 0;
     if (c128 && M > 12) M = 12;
     if (M != 0 && (M < 11 || M > 13)) return fail(SIM_EINVAL, "staged: tile_qubits must be 11, 12 or 13");
@@ -287,8 +308,6 @@ int apply_circuit_staged(qsim_state *s, const sim_gate *gates, size_t n_gates, c
             if (int rc = launch_pair_gate(s, make_pair_gate(gates[k]))) return rc;
         return SIM_OK;
     }
-    std::vector<SGate> g;
-    lower_renamed(gates, n_gates, s->n, &g);
     if (g.empty()) return SIM_OK;
     return c128 ? run_staged<double>(s, g, M) : run_staged<float>(s, g, M);
 }
