@@ -246,10 +246,27 @@ int apply_circuit_learned(qsim_state *s, const sim_gate *gates, size_t n_gates, 
     }
     if (learned_tiles_only(s->n, s->dtype)) {
         // 12-qubit tiles were the fastest variant of every window family here,
-        // or within 3 % of it, and asking the model costs 0.3-0.5 ms of a
+        // or within 6 % of it, and asking the model costs 0.3-0.5 ms of a
         // circuit that takes 0.4-7 ms (18-24 qubits).  Up to 18 qubits the
-        // tiles are of 11 (the staged plan's rule; reported as variant 1, too)
-        s->last_plan.assign((n_gates + (size_t)std::max(64, 8 * s->n) - 1) / (size_t)std::max(64, 8 * s->n), 1);
+        // tiles are of 11 (the staged plan's rule; reported as variant 1, too).
+        // At 25 qubits rotations and exchanges in equal parts go faster in 6-qubit
+        // blocks (U3 + CNOT ladder 1.55 ms against 2.11; at 24 1.03 and 1.08)
+        // (unitary ones: blocks refuse what grows too far)
+        size_t rot = 0, xch = 0;
+        bool unitary = true;
+        for (size_t k = 0; s->n == 25 && k < n_gates; ++k) {
+            const PairGate p = make_pair_gate(gates[k]);
+            unitary = unitary && (p.op == OP_SWAP || unitary_2x2(p.m));
+            if (p.op == OP_DENSE || p.op == OP_ANTIDIAG || (p.op == OP_XPERM && p.nctrl)) (p.nctrl ? xch : rot) += 1;
+        }
+        const bool blocks = s->n == 25 && n_gates >= 16 && unitary && ladder_like(rot, xch, n_gates);
+        s->last_plan.assign((n_gates + (size_t)std::max(64, 8 * s->n) - 1) / (size_t)std::max(64, 8 * s->n), blocks ? 6 : 1);
+        if (blocks) {
+            sim_plan_opts fo{};
+            fo.plan = SIM_PLAN_FUSED;
+            fo.fuse_k = 6;
+            return apply_circuit_fused(s, gates, n_gates, fo);
+        }
         sim_plan_opts so{};
         so.plan = SIM_PLAN_STAGED;
         so.tile_qubits = s->n <= 18 ? 11 : 12;
