@@ -110,7 +110,7 @@ typedef struct sim_plan_opts {
                                 qubits, complex128 from 22): stretches of a unitary circuit that
                                 are predicted to be faster in register tiles run as tile passes. */
     int32_t tile_qubits;     /* SIM_PLAN_STAGED: tile size log2 (0 = default: complex64 11 up to 18
-                                qubits, 12 up to 25, then 13, or 12 where controlled gates that are
+                                qubits, 12 up to 22, then 13, or 12 where controlled gates that are
                                 not X or SWAP, and doubly controlled phases, are more than
                                 an eighth; complex128 11 up to 19, then 12) */
     int32_t flags;           /* SIM_FLAG_* bits, 0 = defaults */

@@ -147,18 +147,18 @@ double tile_cost(const std::vector<SGate> &g, int n, int dtype)
 // The tile size when the caller leaves it open.  Small tiles give small
 // registers more CTAs and shorter programs: 14 qubits, depth-20 random circuit
 // 274 / 307 / 338 us with 11- / 12- / 13-qubit tiles, 18 qubits 385 / 418 / 456, 20
-// qubits 440 / 458 / 500; 22 qubits 839 / 798 / 858.  23 to 25 qubits: 12 and 13 are within
-// 6 % on Haar layers, QFTs, ladders and reversible circuits, and 12 takes a fifth to a
-// quarter less on phases and random gates (24 qubits: 223 / 300 and 814 / 1128 us).  Above, 13
-// saves passes that HBM bounds (28 qubits, Haar layers 13.1 / 12.4 ms, reversible 6.8 / 6.0), except
-// where controlled gates other than moves are more than an eighth: each costs every
-// amplitude a masked multiply, dearer with 64 amplitudes a thread (random gates, 27
-// qubits 7.1 / 9.4 ms, 28 14.0 / 18.2; they took 8.2 and 16.5 before tile programs).
+// qubits 440 / 458 / 500; 22 qubits 839 / 798 / 858.  From 23 on 13: it saves passes that HBM bounds
+// (28 qubits, Haar layers 13.1 / 12.4 ms with 12 / 13, reversible 6.8 / 6.0), which
+// at 23 to 25 is worth nothing yet (the two are within 6 % on Haar layers, QFTs, ladders and reversible
+// circuits there, phases take 223 / 300 us at 24; the learned plan takes 12 up to 25).
+// 12 where controlled gates other than moves, or doubly controlled phases, are more than an eighth:
+// each costs every amplitude a masked multiply, dearer with 64 amplitudes a thread (random gates, 24
+// qubits 0.81 / 1.13 ms, 27 7.1 / 9.4, 28 14.0 / 18.2; 1.06, 8.2 and 16.5 before tile programs).
 // complex128: 12 qubits wherever they fit (26-qubit QFT 24.3 against 25.3 ms).
 static int open_tile(const std::vector<SGate> &g, int n, bool c128)
 {
     if (c128) return n >= 20 ? 12 : 11;
-    if (n <= 25) return n <= 18 ? 11 : 12;
+    if (n <= 22) return n <= 18 ? 11 : 12;
     size_t masked = 0;
     for (const SGate &x : g)
         masked += x.xq() ? x.ctrl && x.op != OP_XPERM && x.op != OP_SWAP : __builtin_popcountll(x.ctrl) >= 2;
