@@ -108,7 +108,8 @@ typedef struct sim_plan_opts {
                                 the fixed-point rounding).  Every fused plan needs
                                 n >= k + 7 (SIM_EINVAL otherwise).  Large registers (k = 6 from 26
                                 qubits, complex128 from 22): stretches of a unitary circuit that
-                                are predicted to be faster in register tiles run as tile passes. */
+                                are predicted to be faster in register tiles run as tile passes (a
+                                circuit with a matrix that is not unitary to 1e-6 runs in blocks). */
     int32_t tile_qubits;     /* SIM_PLAN_STAGED: tile size log2 (0 = default: complex64 11 up to 18
                                 qubits, 12 up to 22, then 13, or 12 where controlled gates that are
                                 not X or SWAP, and doubly controlled phases, are more than
@@ -341,14 +342,17 @@ int sim_batch_destroy(sim_batch_t b);
  *   eps 1e-8, learning rate lr); *final_loss (may be NULL) after the last.
  * sim_set_cost_model: SIM_PLAN_LEARNED on this handle consults model m (NULL
  *   = no model: the greedy fixed-k plan is used).  The model must outlive the
- *   handle's use of it.  Registers of 12 to 25 qubits run 12-qubit register
- *   tiles without asking it (fastest, or within 3 %, on every circuit family;
- *   asking costs more than that); from 26 qubits on it is asked about the windows that
- *   controlled exchanges decide, the others run as the fused plan with k = 6,
- *   which takes tile passes where they are faster.  A complex128 handle runs SIM_PLAN_LEARNED without
- *   consulting the model (trained on complex64 timings): as the fused plan
- *   with k = 4 when n >= 11 (tensor-core digit products; the per-gate and
- *   register-tile kernels are bound by the FP64 pipe), else per gate. */
+ *   handle's use of it.  Registers of 12 to 25 qubits run register tiles (of 11
+ *   qubits up to 18, then of 12) without asking it (fastest, or within 6 %, on almost every
+ *   circuit family; asking costs more than that), except that at 25 qubits circuits of rotations and
+ *   controlled exchanges in about equal parts run 6-qubit blocks; from 26 qubits on it
+ *   is asked about the windows that controlled exchanges decide, the others run as
+ *   the fused plan with k = 6, which takes tile passes where they are faster.  A
+ *   complex128 handle runs SIM_PLAN_LEARNED without consulting the model
+ *   (trained on complex64 timings): from 11 qubits as the fused plan with k = 4 in its
+ *   mixed form (4-qubit blocks of tensor-core digit products, or tile passes where they are
+ *   faster: up to 19 qubits tiles unless controlled dense gates are more than a third;
+ *   circuits that are not unitary run in blocks), below per gate. */
 typedef struct qsim_mlp *sim_mlp_t;
 int sim_mlp_param_count(int d_in, int hidden);
 int sim_mlp_create(int d_in, int hidden, void *stream, sim_mlp_t *out);
@@ -370,7 +374,11 @@ int sim_set_cost_model(sim_t s, sim_mlp_t m);
 #define SIM_VARIANTS 7
 int sim_plan_features(int n, int dtype, const sim_gate *gates, size_t n_gates, int variant, float *out);
 /* sim_last_plan: the variant the last SIM_PLAN_LEARNED call chose for each
- *   window of gates (up to cap entries; the count in *len). */
+ *   window of gates (up to cap entries; the count in *len).  It names the choice, not
+ *   every kernel: 1 stands for register tiles without asking the model (of 11
+ *   qubits up to 18), 2 for the staged plan with its open tile size,
+ *   6 from 26 qubits and complex128's single entry 4 for the fused plan in its
+ *   mixed form, which may run all of it in tile passes. */
 int sim_last_plan(sim_t s, int32_t *variants, size_t cap, size_t *len);
 
 /* ---- plan introspection (host only, no GPU needed) ---------------------------

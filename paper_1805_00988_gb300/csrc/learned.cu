@@ -24,7 +24,7 @@ namespace qsim {
 
 namespace {
 
-constexpr int kConsultFrom = 26;   // complex64 registers below run 12-qubit tiles without asking the model
+constexpr int kConsultFrom = 26;   // complex64 registers below run tiles without asking the model
 
 struct Window {
     size_t first, count;
@@ -102,7 +102,10 @@ int learned_choose(qsim_state *s, const sim_gate *gates, size_t n_gates, std::ve
     for (size_t f = 0; f < n_gates; f += W) win.push_back(Window{f, std::min(W, n_gates - f)});
     const size_t nw = win.size();
     // predicted log times of the feasible variants of some segments, the
-    // feature rows in parallel on the host threads, one batched forward pass
+    // feature rows in parallel on the host threads, one batched forward pass.
+    // The shipped weights are of timings before tile programs and the mixed plan, and
+    // the features still count the record schedule: what is left to the model are the
+    // windows below, and tiles are twice as fast as it knows
     // where the 6-qubit fused plan mixes in tile passes it holds the other
     // variants' strengths: only the 13-qubit tile plan is weighed against it,
     // and has to be predicted faster by more than the model's error
@@ -226,12 +229,12 @@ int apply_circuit_learned(qsim_state *s, const sim_gate *gates, size_t n_gates, 
         // complex128: the per-gate and register-tile kernels are bound by this
         // GPU's narrow FP64 pipe, while 4-qubit fused blocks run on the FP16
         // tensor cores as exact integer digit-plane products (fused64.cu).
-        // Measured at 30 qubits (Haar layers + CZ, depth 20): fused 1276 ms
-        // against 12837 ms per gate; 28-qubit QFT: 253 against 351 ms.  So the
-        // fused plan, with register tiles where those are faster (its mixed
-        // form), runs wherever a 4-qubit block's tile fits (n >= 11), the
+        // Measured at 30 qubits (Haar layers + CZ, depth 20): blocks 769 ms
+        // against 10400 ms per gate; 28-qubit QFT: mixed 105 against 265 ms.  So the
+        // fused plan in its mixed form (register tiles where those are faster, up to 19
+        // qubits almost always) runs wherever a 4-qubit block's tile fits (n >= 11), the
         // per-gate plan below that; the model (trained on complex64 timings)
-        // is not consulted.
+        // is not consulted.  Reported as variant 4.
         if (s->n >= 11) {
             s->last_plan.assign(1, 4);
             sim_plan_opts fo{};

@@ -363,7 +363,8 @@ __global__ void __launch_bounds__(kRedThreads) k_masked_sum(const R *__restrict_
 // amplitudes) one power-of-two scale, two carries into FP64 (8 amplitudes
 // each).  The batches, the grid and the FP64 tree are those of k_masked_sum.
 // RED_BIT: bit q is usually the same for all of a thread's batch, which then needs
-// no choice of sum per amplitude (28 qubits: 0.43 -> 0.38 ms, the same bits).
+// no choice of sum per amplitude (28 qubits: 0.43 -> 0.38 ms; the batch's two carries are added
+// to each other first, so the last bit can differ from the path below).
 template <int MODE>
 __global__ void __launch_bounds__(kRedThreads) k_sum_sq32(const float *__restrict__ st, uint64_t nvec, uint64_t per,
                                                           int q, double *__restrict__ partial)

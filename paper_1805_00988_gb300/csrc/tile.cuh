@@ -1,6 +1,7 @@
 // tile.cuh -- register layouts of a tile, the host pass planner, and the
-// record schedule of a pass (what sim_plan_describe and sim_plan_staged_ops
-// report, for 256 threads a tile).  What the kernels run is compiled from the
+// record schedule of a pass (for 256 threads a tile).  No kernel runs the records: the cost
+// model's features count them, and sim_plan_describe (all but its passes) and
+// sim_plan_staged_ops report them.  What the kernels run is compiled from the
 // passes by tileprog.cuh.  See staged.cu for the design.
 #pragma once
 
