@@ -240,7 +240,7 @@ constexpr int kThreads = 256;
 // with 512-pair blocks, 5.5 with 64; 20 qubits 12.6 and 11.3; from 21 on, and for
 // controlled and diagonal gates from 20 on, the big ones win).
 constexpr int kSmallThreads = 64;
-constexpr uint64_t kSpread = 152, kSpread64 = 608, kSpreadDense64 = 1216;
+constexpr uint64_t kSpread = 1, kSpread64 = 4, kSpreadDense64 = 8;     // blocks per SM
 
 __device__ __forceinline__ void pdl_enter()
 {
@@ -344,7 +344,7 @@ template <typename R, int VEC, int OP, int U>
 void go_split(qsim_state *s, const PairArgs &a, const Coef<R> &c)
 {
     const uint64_t per = (uint64_t)kThreads * U, blocks = (a.n_items + per - 1) / per;
-    if (blocks >= (sizeof(R) == 4 ? kSpread : OP == OP_DENSE ? kSpreadDense64 : kSpread64))
+    if (blocks >= (sizeof(R) == 4 ? kSpread : OP == OP_DENSE ? kSpreadDense64 : kSpread64) * (uint64_t)s->num_sms)
         launch_pdl(s->stream, k_pair_split<R, VEC, OP, U>, blocks, kThreads, (R *)s->amps, a, c);
     else
         launch_pdl(s->stream, k_pair_split<R, VEC, OP, 1>, (a.n_items + kSmallThreads - 1) / kSmallThreads,
@@ -356,7 +356,7 @@ void go_inner(qsim_state *s, const PairArgs &a, const Coef<float> &c)
 {
     constexpr int U = 4;
     const uint64_t per = (uint64_t)kThreads * U, blocks = (a.n_items + per - 1) / per;
-    if (blocks >= kSpread)
+    if (blocks >= kSpread * (uint64_t)s->num_sms)
         launch_pdl(s->stream, k_pair_inner<OP, U>, blocks, kThreads, (float *)s->amps, a, c);
     else
         launch_pdl(s->stream, k_pair_inner<OP, 1>, (a.n_items + kSmallThreads - 1) / kSmallThreads, kSmallThreads,
