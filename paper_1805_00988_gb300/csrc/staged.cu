@@ -297,7 +297,7 @@ int apply_circuit_staged(qsim_state *s, const sim_gate *gates, size_t n_gates, c
 {
     const bool c128 = s->dtype == SIM_C128;
     std::vector<SGate> g;
-    lower_renamed(gates, n_gates, s->n, &g);
+    if (s->n >= 11) lower_renamed(gates, n_gates, s->n, &g);
     int M = o.tile_qubits ? o.tile_qubits : open_tile(g, s->n, c128);
     if (M > s->n) M = (s->n >= 11) ? 11 : 0;
     if (c128 && M > 12) M = 12;
